@@ -116,12 +116,12 @@ typedef struct {
   amr_face faces[6];       /* x-, x+, y-, y+, z-, z+ (first 4 used in 2D)      */
   int32_t use_graphs;      /* 1: replay the coarse step as a CUDA graph         */
   int32_t kernel_variant;  /* collide-stream kernel (fused BGK + pull
-                              streaming): 1 / 2 / 3 / 4: 512 / 256 / 128 /
-                              64 threads per CTA (8 / 4 / 2 / 1 blocks in 3D);
-                              5: 128 threads with 512 more resident threads
-                              per SM (tighter register budget); 0 (default):
-                              64 threads, with the tighter budget for D3Q27
-                              with 16-bit storage                              */
+                              streaming): 1 / 2 / 3 / 4: CTAs of 512 / 256 /
+                              128 / 64 cells (8 / 4 / 2 / 1 blocks in 3D; at
+                              least the blocks of one warp); 5: 128 cells with
+                              128 more resident threads per SM (tighter
+                              register budget); 0 (default): 256 cells in 3D,
+                              64 in 2D, 32 in 2D FP64                        */
   double refine_dist;      /* distance refinement (Section 4.4): a leaf on level
                               L within refine_dist / 2^L (physical units) of a
                               target is marked for refinement; 0 = off        */
@@ -480,8 +480,9 @@ int amr_propose_marks(amr_t* a, const void* params_half, float threshold, int wi
  *   timeout the persistent form does nothing until amr_batch_sync has
  *   reported it; the members' populations are then part-way through a step.
  * amr_batch_configure: select the form and its tile shape.  Graph form:
- *   threads per CTA of the batched collide-stream 64, 128, 256 or 512 (the
- *   CTA takes threads / 4^D blocks); tile_blocks and ctas are ignored.
+ *   threads = cells per CTA of the batched collide-stream, 64, 128, 256 or
+ *   512 (the CTA takes threads / 4^D blocks, at least those of one warp);
+ *   tile_blocks and ctas are ignored.
  *   Persistent form: threads 64, 128 or 256 per CTA, tile_blocks M_L = 1..8
  *   blocks per collide-stream tile (an interpolation or averaging tile holds
  *   threads / 4^D parents or children), ctas = CTAs launched (0: as many as

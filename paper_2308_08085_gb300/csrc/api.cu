@@ -296,6 +296,7 @@ static void collide_stream_level(Instance* a, int L, bool ghost_in, const Exchan
   }
   StepParams prm = a->prm;
   prm.omega = 1.0 / a->tau[L];
+  prm.omega32 = (float)prm.omega;
   double bytes = (double)n * a->M * 2.0 * a->q * a->elem;
   if (xchg) bytes += (double)a->n_ghost_cells[L] * a->q * a->elem;   // ghost cells written
   {
@@ -337,6 +338,7 @@ static void advance(Instance* a, int L, bool first) {
     ex.child0 = a->child0;
     ex.cellmask = a->cellmask;
     ex.r_cf = ratio_cf(a, L);
+    ex.keep32 = (float)(1.0 - ex.r_cf);
   }
   collide_stream_level(a, L, first && L > 0 && a->n_parents[L - 1] > 0, xchg ? &ex : nullptr);
   if (fine) {
@@ -670,9 +672,11 @@ int amr_init(const amr_config* cfg, void* arena, size_t arena_bytes, void* strea
     a->prm.faces.kind[f] = fc.kind;
     const double rho_w = fc.rho_w > 0 ? fc.rho_w : 1.0;
     a->prm.faces.rho_w[f] = rho_w;
+    a->prm.faces.rho_w32[f] = (float)rho_w;
     for (int p = 0; p < a->q; ++p) {
       const double cu = c[p][0] * fc.u[0] + c[p][1] * fc.u[1] + (a->dim == 3 ? c[p][2] * fc.u[2] : 0.0);
       a->prm.faces.bb[f][p] = fc.kind == AMR_FACE_MOVING ? -2.0 * w[p] * rho_w * cu * 3.0 : 0.0;
+      a->prm.faces.bb32[f][p] = (float)a->prm.faces.bb[f][p];
     }
   }
   int rc = AMR_OK;

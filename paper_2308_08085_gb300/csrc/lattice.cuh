@@ -119,12 +119,16 @@ template <class T> struct Store;
 template <> struct Store<double> {
   using R = double;
   static constexpr bool kShifted = false;
+  __device__ static R raw(double v) { return v; }
+  __device__ static double from_raw(R v) { return v; }
   template <int D, int Q, int P> __device__ static R load(double v) { return v; }
   template <int D, int Q, int P> __device__ static double save(R v) { return v; }
 };
 template <> struct Store<float> {
   using R = float;
   static constexpr bool kShifted = false;
+  __device__ static R raw(float v) { return v; }
+  __device__ static float from_raw(R v) { return v; }
   template <int D, int Q, int P> __device__ static R load(float v) { return v; }
   template <int D, int Q, int P> __device__ static float save(R v) { return v; }
 };

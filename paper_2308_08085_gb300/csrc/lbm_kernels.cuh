@@ -473,80 +473,28 @@ __global__ void __launch_bounds__(128, 8)
 // ================================================ batched instances (lock-step)
 // Work items pack (instance, block) as inst << BATCH_SHIFT | block; each
 // instance's buffers, tables and per-level factors come from its descriptor.
-// The same pull step as k_collide_stream (no solid cells in a batch).
+// The same step as k_collide_stream (no solid cells in a batch).
 template <int D, int Q, class T, int THREADS>
-__global__ void __launch_bounds__(THREADS, (one_pass_min_blocks<T, Q, THREADS>()))
+__global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
     k_collide_stream_batch(const uint32_t* __restrict__ items, int n,
                            const InstDesc* __restrict__ descs, int level, int which_in) {
-  using S = Store<T>;
-  using R = typename S::R;
-  constexpr int M = Block<D>::M;
-  constexpr int NCODE = D == 2 ? 9 : 27;
-  constexpr int CENTER = D == 2 ? 4 : 13;
-  constexpr int BPC = THREADS / M;
-  __shared__ int32_t s_nb[BPC][NCODE];
-  __shared__ int32_t s_inst[BPC];
-  const int slot = threadIdx.x / M;
-  const int l = threadIdx.x - slot * M;
-  const int first = blockIdx.x * BPC;
-  for (int t = threadIdx.x; t < BPC * NCODE; t += THREADS) {
-    const int s = t / NCODE, code = t - s * NCODE;
-    const int bi = first + s;
-    int v = NONE;
-    if (bi < n) {
-      const uint32_t it = __ldg(items + bi);
-      const int inst = (int)(it >> BATCH_SHIFT);
-      const int b = (int)(it & BATCH_MASK);
-      v = __ldg(descs[inst].nbr + (size_t)b * NBR_STRIDE + geo_to_k<D>(code));
-      if (code == 0) s_inst[s] = inst;
-    }
-    s_nb[s][code] = v;
-  }
-  __syncthreads();
-  int flags;
-  {
-    const int v = s_nb[slot][l % NCODE];
-    const unsigned lanes = M >= 32 ? 0xffffffffu : (((1u << M) - 1u) << ((threadIdx.x & 31) & ~(M - 1)));
-    const unsigned outside = __ballot_sync(0xffffffffu, v < 0) & lanes;
-    // (a slot past the end of the list has only NONE entries: no descriptor read)
-    const unsigned wall = __ballot_sync(
-        0xffffffffu, v <= -2 && descs[s_inst[slot]].faces.kind[-2 - v] != FACE_NOSLIP) & lanes;
-    const unsigned outlet = __ballot_sync(
-        0xffffffffu, v <= -2 && descs[s_inst[slot]].faces.kind[-2 - v] == FACE_OUTLET) & lanes;
-    flags = (outside ? BF_OUTSIDE : 0) | (wall ? BF_WALL : 0) | (outlet ? BF_OUTLET : 0);
-  }
-  if (first + slot >= n) return;
-  const InstDesc& d = descs[s_inst[slot]];
-  const int b = s_nb[slot][CENTER];
-  const T* __restrict__ gin = (const T*)d.f[which_in];
-  T* __restrict__ gout = (T*)d.f[which_in ^ 1];
-  const size_t own = (size_t)b * (Q * M) + l;
-  const int32_t* nb = s_nb[slot];
-  if (flags == 0) {
-    R f[Q];
-    static_for<0, Q>([&](auto P) {
-      constexpr int p = P;
-      if constexpr (p == 0) {
-        f[0] = S::template load<D, Q, 0>(gin[own]);
-      } else {
-        const int e = link_entry<D, Q, p>(g_src_geo<D, Q>, l);
-        f[p] = S::template load<D, Q, p>(
-            gin[(size_t)nb[e & 31] * (Q * M) + (size_t)p * M + (e >> 5)]);
-      }
-    });
-    R ux, uy, uz, usq15;
-    bgk<D, Q>(f, R(d.omega[level]), ux, uy, uz, usq15);
-    static_for<0, Q>([&](auto P) {
-      gout[own + (size_t)P * M] = S::template save<D, Q, P>(f[P]);
-    });
-  } else {
-    if (flags & BF_OUTLET)
-      step_cell_checked<D, Q, T, false, true>(gin, gout, own, l, nb, nullptr, flags,
-                                              d.omega[level], d.faces, false);
-    else
-      step_cell_checked<D, Q, T, false, false>(gin, gout, own, l, nb, nullptr, flags,
-                                               d.omega[level], d.faces, false);
-  }
+  using R = typename Store<T>::R;
+  constexpr int V = row_cells<D, T>();
+  constexpr int TPB = Block<D>::M / V;
+  constexpr int BPC = THREADS / TPB;
+  __shared__ int32_t s_nb[BPC][D == 2 ? 9 : 27];
+  const int slot = threadIdx.x / TPB;
+  const int t = threadIdx.x % TPB;
+  const int bi = blockIdx.x * BPC + slot;
+  if (bi >= n) return;
+  const uint32_t it = __ldg(items + bi);
+  const InstDesc& d = descs[it >> BATCH_SHIFT];
+  const int b = (int)(it & BATCH_MASK);
+  const int flags = stage_block<D, TPB, false>(s_nb[slot], nullptr, b, t, block_lanes<TPB>(),
+                                               d.nbr, nullptr, d.faces);
+  step_row<D, Q, T, V, false, false, false, false>(
+      (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[slot], nullptr, flags, 0ull,
+      R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
 }
 
 template <int D, int Q, class T>
@@ -642,67 +590,23 @@ __device__ __forceinline__ bool persist_wait(const uint32_t* cnt, uint32_t targe
 }
 
 // Collide-stream tile: `nblk` (<= PERSIST_MAX_TILE) active blocks of one
-// member, the cells spread over the CTA's threads.  The same pull step as
+// member, their rows spread over the CTA's threads.  The same step as
 // k_collide_stream_batch, with every population read from L2.
 template <int D, int Q, class T, int THREADS>
 __device__ __forceinline__ void persist_collide(const InstDesc& d, const uint32_t* items, int nblk,
                                                 int level, int which_in,
-                                                int32_t (*s_nb)[D == 2 ? 9 : 27],
-                                                int32_t* s_flags) {
-  using S = Store<T>;
-  using R = typename S::R;
-  constexpr int M = Block<D>::M;
-  constexpr int NCODE = D == 2 ? 9 : 27;
-  constexpr int CENTER = D == 2 ? 4 : 13;
-  for (int e = threadIdx.x; e < nblk * NCODE; e += THREADS) {
-    const int s = e / NCODE, code = e - s * NCODE;
+                                                int32_t (*s_nb)[D == 2 ? 9 : 27]) {
+  using R = typename Store<T>::R;
+  constexpr int V = row_cells<D, T>();
+  constexpr int TPB = Block<D>::M / V;
+  const int t = threadIdx.x % TPB;
+  for (int s = threadIdx.x / TPB; s < nblk; s += THREADS / TPB) {
     const int b = (int)(__ldg(items + s) & BATCH_MASK);
-    s_nb[s][code] = __ldg(d.nbr + (size_t)b * NBR_STRIDE + geo_to_k<D>(code));
-  }
-  __syncthreads();
-  if (threadIdx.x < nblk) {
-    int flags = 0;
-    for (int code = 0; code < NCODE; ++code) {
-      const int v = s_nb[threadIdx.x][code];
-      if (v < 0) flags |= BF_OUTSIDE;
-      if (v <= -2 && d.faces.kind[-2 - v] != FACE_NOSLIP) flags |= BF_WALL;
-      if (v <= -2 && d.faces.kind[-2 - v] == FACE_OUTLET) flags |= BF_OUTLET;
-    }
-    s_flags[threadIdx.x] = flags;
-  }
-  __syncthreads();
-  const T* gin = (const T*)d.f[which_in];
-  T* gout = (T*)d.f[which_in ^ 1];
-  const double omega = d.omega[level];
-  for (int c = threadIdx.x; c < nblk * M; c += THREADS) {
-    const int s = c / M, l = c - s * M;
-    const int32_t* nb = s_nb[s];
-    const size_t own = (size_t)nb[CENTER] * (Q * M) + l;
-    const int flags = s_flags[s];
-    if (flags == 0) {
-      R f[Q];
-      static_for<0, Q>([&](auto P) {
-        constexpr int p = P;
-        if constexpr (p == 0) {
-          f[0] = S::template load<D, Q, 0>(__ldcg(gin + own));
-        } else {
-          const int e = link_entry<D, Q, p>(g_src_geo<D, Q>, l);
-          f[p] = S::template load<D, Q, p>(
-              __ldcg(gin + (size_t)nb[e & 31] * (Q * M) + (size_t)p * M + (e >> 5)));
-        }
-      });
-      R ux, uy, uz, usq15;
-      bgk<D, Q>(f, R(omega), ux, uy, uz, usq15);
-      static_for<0, Q>([&](auto P) {
-        gout[own + (size_t)P * M] = S::template save<D, Q, P>(f[P]);
-      });
-    } else if (flags & BF_OUTLET) {
-      step_cell_checked<D, Q, T, false, true, false, true>(gin, gout, own, l, nb, nullptr,
-                                                           flags, omega, d.faces, false);
-    } else {
-      step_cell_checked<D, Q, T, false, false, false, true>(gin, gout, own, l, nb,
-                                                            nullptr, flags, omega, d.faces, false);
-    }
+    const int flags = stage_block<D, TPB, false>(s_nb[s], nullptr, b, t, block_lanes<TPB>(),
+                                                 d.nbr, nullptr, d.faces);
+    step_row<D, Q, T, V, false, false, false, true>(
+        (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[s], nullptr, flags, 0ull,
+        R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
   }
 }
 
@@ -768,7 +672,7 @@ __device__ __noinline__ void persist_average(const InstDesc& d, const uint32_t* 
 // the THREADS / M parents (interpolation) or children (averaging) of a tile,
 // then their neighbour rows.
 template <int D, int Q, class T, int THREADS>
-__global__ void __launch_bounds__(THREADS, (one_pass_min_blocks<T, Q, THREADS>()))
+__global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
     k_batch_persistent(PersistArgs a) {
   using R = typename Store<T>::R;
   constexpr int M = Block<D>::M;
@@ -780,7 +684,6 @@ __global__ void __launch_bounds__(THREADS, (one_pass_min_blocks<T, Q, THREADS>()
   int32_t (*s_rows)[1 + NC][NK] =
       reinterpret_cast<int32_t (*)[1 + NC][NK]>(s_dyn + sizeof(R) * U * Q * M);
   __shared__ int32_t s_nb[PERSIST_MAX_TILE][D == 2 ? 9 : 27];
-  __shared__ int32_t s_flags[PERSIST_MAX_TILE];
   __shared__ long long s_take;
   __shared__ int32_t s_go;
   const long long total = (long long)a.tiles_per_step * a.n_steps;
@@ -846,7 +749,7 @@ __global__ void __launch_bounds__(THREADS, (one_pass_min_blocks<T, Q, THREADS>()
     if (op == PH_COLLIDE) {
       const int first = tile * a.tile_blocks;
       const int nblk = min(a.tile_blocks, ni - first);
-      persist_collide<D, Q, T, THREADS>(d, items + first, nblk, level, win, s_nb, s_flags);
+      persist_collide<D, Q, T, THREADS>(d, items + first, nblk, level, win, s_nb);
     } else if (op == PH_INTERP) {
       persist_interp<D, Q, T, THREADS>(d, items, ni, tile, level, win, wch, sF, s_rows);
     } else {
@@ -1293,6 +1196,10 @@ template <int D, int Q, class T>
 struct Launch {
   static constexpr int M = Block<D>::M;
   static inline int sm_count = 152;
+  // cells per CTA.  2D meshes are small: CTAs of one or two warps spread them
+  // over the SMs (an SM executes one FP64 warp instruction per 19 cycles; the
+  // 64^2 FP64 cavity took 2.20 ms with 256 cells per CTA, 1.66 with 32)
+  static constexpr int kAutoCells = D == 3 ? 256 : (sizeof(T) == 8 ? 32 : 64);
 
   static int setup() {
     int dev = 0, sms = 0;
@@ -1302,43 +1209,39 @@ struct Launch {
     return 0;
   }
 
-  template <bool SOLID, int THREADS, bool DENSE = false>
+  // CELLS cells per CTA (at least the blocks of a warp)
+  template <bool SOLID, int CELLS, bool DENSE = false>
   static void one_pass(cudaStream_t s, const int32_t* list, int n, const void* fin, void* fout,
                        const int32_t* nbr, const uint64_t* sm, const StepParams& prm,
                        const uint64_t* gm, const Exchange* xchg) {
-    const int grid = grid_for(n, THREADS / M);
+    constexpr int THREADS = row_threads<D, T>(CELLS);
+    constexpr int MIN = row_min_ctas<Q, T, THREADS, DENSE>();
     const T* in = (const T*)fin;
     T* out = (T*)fout;
     Exchange ex{};
     if (xchg) ex = *xchg;
-    if (gm && xchg)
-      k_collide_stream<D, Q, T, SOLID, THREADS, DENSE, true, true>
+    auto launch = [&](auto ghost, auto parents) {
+      constexpr bool G = decltype(ghost)::value, X = decltype(parents)::value;
+      const int grid = grid_for(n, THREADS * row_cells<D, T>() / M);
+      k_collide_stream<D, Q, T, SOLID, THREADS, MIN, G, X>
           <<<grid, THREADS, 0, s>>>(list, n, in, out, nbr, sm, prm, gm, ex);
-    else if (gm)
-      k_collide_stream<D, Q, T, SOLID, THREADS, DENSE, true, false>
-          <<<grid, THREADS, 0, s>>>(list, n, in, out, nbr, sm, prm, gm, ex);
-    else if (xchg)
-      k_collide_stream<D, Q, T, SOLID, THREADS, DENSE, false, true>
-          <<<grid, THREADS, 0, s>>>(list, n, in, out, nbr, sm, prm, nullptr, ex);
-    else
-      k_collide_stream<D, Q, T, SOLID, THREADS, DENSE, false, false>
-          <<<grid, THREADS, 0, s>>>(list, n, in, out, nbr, sm, prm, nullptr, ex);
+    };
+    if (gm && xchg) launch(std::true_type{}, std::true_type{});
+    else if (gm) launch(std::true_type{}, std::false_type{});
+    else if (xchg) launch(std::false_type{}, std::true_type{});
+    else launch(std::false_type{}, std::false_type{});
   }
 
   template <bool SOLID>
   static void collide_stream_t(cudaStream_t s, const int32_t* list, int n, const void* fin,
                                void* fout, const int32_t* nbr, const uint64_t* sm,
                                const StepParams& prm, const uint64_t* gm, const Exchange* x) {
-    // kernel_variant: 1 / 2 / 3 / 4: 512 / 256 / 128 / 64 threads per CTA
-    // (8 / 4 / 2 / 1 blocks of 4^3 cells); 5: 128 threads with 512 more
-    // resident threads per SM (tighter register budget); 0 (auto): 64
-    // threads (the fastest in the 3D cavity's AMR step, where the blocks of
-    // a CTA take different paths), with the tighter budget for D3Q27 with
-    // 16-bit storage.  Launches with exchanging parents always run 64
-    // threads per CTA, so that a parent's barrier holds no other block.
-    constexpr bool kDenseAuto = Q == 27 && sizeof(T) == 2;
-    if (x) {
-      one_pass<SOLID, 64, kDenseAuto>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
+    // kernel_variant: 1 / 2 / 3 / 4: CTAs of 512 / 256 / 128 / 64 cells (8 /
+    // 4 / 2 / 1 blocks of 4^3 cells; never less than a warp); 5: 128 cells
+    // with 128 more resident threads per SM (tighter register budget); 0
+    // (auto) and launches with exchanging parents: kAutoCells
+    if (x || prm.variant == 0 || prm.variant > 5) {
+      one_pass<SOLID, kAutoCells>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
       return;
     }
     switch (prm.variant) {
@@ -1347,7 +1250,6 @@ struct Launch {
       case 3: one_pass<SOLID, 128>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 4: one_pass<SOLID, 64>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 5: one_pass<SOLID, 128, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      default: one_pass<SOLID, 64, kDenseAuto>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr);
     }
   }
 
@@ -1468,25 +1370,22 @@ struct Launch {
   static void collide_stream_batch(cudaStream_t s, const uint32_t* items, int n,
                                    const InstDesc* descs, int level, int which_in, int variant) {
     if (n <= 0) return;
-    // variant = threads per CTA: 64 / 128 / 256 / 512, i.e. M_L = 64/M .. 512/M
-    // blocks per CTA (anything else: 512)
+    // variant: 64 / 128 / 256 / 512 cells per CTA, i.e. M_L = 64/M .. 512/M
+    // blocks (never less than a warp; anything else: 512)
     switch (variant) {
-      case 64:
-        k_collide_stream_batch<D, Q, T, 64><<<grid_for(n, 64 / M), 64, 0, s>>>(items, n, descs,
-                                                                              level, which_in);
-        break;
-      case 128:
-        k_collide_stream_batch<D, Q, T, 128><<<grid_for(n, 128 / M), 128, 0, s>>>(
-            items, n, descs, level, which_in);
-        break;
-      case 256:
-        k_collide_stream_batch<D, Q, T, 256><<<grid_for(n, 256 / M), 256, 0, s>>>(
-            items, n, descs, level, which_in);
-        break;
-      default:
-        k_collide_stream_batch<D, Q, T, 512><<<grid_for(n, 512 / M), 512, 0, s>>>(
-            items, n, descs, level, which_in);
+      case 64: batch_cells<64>(s, items, n, descs, level, which_in); break;
+      case 128: batch_cells<128>(s, items, n, descs, level, which_in); break;
+      case 256: batch_cells<256>(s, items, n, descs, level, which_in); break;
+      default: batch_cells<512>(s, items, n, descs, level, which_in);
     }
+  }
+  template <int CELLS>
+  static void batch_cells(cudaStream_t s, const uint32_t* items, int n, const InstDesc* descs,
+                          int level, int which_in) {
+    constexpr int THREADS = row_threads<D, T>(CELLS);
+    k_collide_stream_batch<D, Q, T, THREADS>
+        <<<grid_for(n, THREADS * row_cells<D, T>() / M), THREADS, 0, s>>>(items, n, descs, level,
+                                                                          which_in);
   }
   static void interp_batch(cudaStream_t s, const uint32_t* items, int n, const InstDesc* descs,
                            int level, int which_par, int which_ch) {

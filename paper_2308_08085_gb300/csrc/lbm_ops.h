@@ -12,6 +12,16 @@ struct FaceParams {
   int32_t kind[6];      // AMR_FACE_*
   double rho_w[6];
   double bb[6][27];     // bounce-back term -2 w_p rho_w (c_p . u_w) / cs^2
+  float rho_w32[6];     // the same in FP32: an FP64 conversion or product in a
+  float bb32[6][27];    // kernel occupies a scheduler for 64 cycles
+  template <class R> __host__ __device__ R rho(int face) const {
+    if constexpr (sizeof(R) == 8) return rho_w[face];
+    else return rho_w32[face];
+  }
+  template <class R> __host__ __device__ R link(int face, int p) const {
+    if constexpr (sizeof(R) == 8) return bb[face][p];
+    else return bb32[face][p];
+  }
 };
 
 // Descriptor of one instance inside a batch (Section 4.1 level step applied to
@@ -83,13 +93,23 @@ struct Exchange {
   const int32_t* child0;
   const uint64_t* cellmask;    // [2 b]: ghost cells, [2 b + 1]: interface cells
   double r_cf;                 // coarse -> fine rescale, tau_F / (2 tau_C)
+  float keep32;                // 1 - r_cf in FP32
+  template <class R> __host__ __device__ R keep() const {
+    if constexpr (sizeof(R) == 8) return 1.0 - r_cf;
+    else return keep32;
+  }
 };
 
 struct StepParams {
   double omega;         // 1 / tau_L
+  float omega32;        // the same in FP32
   int variant;          // collide-stream kernel variant (amr_config.kernel_variant)
   FaceParams faces;
   int32_t* wait_flag;   // device int set to 1 by a kernel whose bounded wait gave up
+  template <class R> __host__ __device__ R rate() const {
+    if constexpr (sizeof(R) == 8) return omega;
+    else return omega32;
+  }
 };
 
 // Every kernel reads the populations of a cell through the gather and writes
