@@ -357,10 +357,10 @@ static void advance(Instance* a, int L, bool first) {
       if (cubic)
         a->ops->average(a->stream, a->parents + (size_t)L * a->cap, (int)np, true,
                         a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                        a->cellmask, a->status, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
+                        a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
       else
         a->ops->average_groups(a->stream, a->agrp + a->agrp_off[L + 1], (int)a->n_agrp[L + 1],
-                               a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0,
+                               a->fbuf(L, 0), a->fbuf(L + 1, 0), a->n_root,
                                a->parent, a->nbr, a->sm(), ratio_fc(a, L), a->solid);
       a->launches += 1;
     }
@@ -449,9 +449,10 @@ static int build_graphs(Handle* h) {
 static void level_sync(Instance* a) {
   for (int L = a->lmax - 2; L >= 0; --L) {
     if (a->n_ids[L + 1] == 0) continue;
-    a->ops->average(a->stream, a->idset + (size_t)L * a->cap, (int)a->n_ids[L], true,
+    // every block of level L + 1 is the child of a refined block
+    a->ops->average(a->stream, a->order + (size_t)(L + 1) * a->cap, (int)a->n_ids[L + 1], false,
                     a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                    a->cellmask, a->status, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
+                    a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
     a->launches += 1;
   }
   for (int L = 0; L + 1 < a->lmax; ++L) {

@@ -592,11 +592,12 @@ __device__ __forceinline__ unsigned block_lanes() {
 // The TPB threads of a block stage its neighbour row in geometric order (and
 // the solid cells of those blocks) in shared memory and return the block's
 // flags to every one of them.  `lanes`: their bits within the warp.
+// (faces null: the walls are not looked at)
 template <int D, int TPB, bool SOLID>
 __device__ __forceinline__ int stage_block(int32_t* s_nb, uint64_t* s_sm, int b, int t,
                                            unsigned lanes, const int32_t* __restrict__ nbr,
                                            const uint64_t* __restrict__ solidmask,
-                                           const FaceParams& faces) {
+                                           const FaceParams* faces) {
   constexpr int NCODE = D == 2 ? 9 : 27;
   int flags = 0;
   const int32_t* row = nbr + (size_t)b * NBR_STRIDE;
@@ -607,7 +608,7 @@ __device__ __forceinline__ int stage_block(int32_t* s_nb, uint64_t* s_sm, int b,
       const int v = __ldg(row + geo_to_k<D>(code));
       s_nb[code] = v;
       if (v < 0) flags |= BF_OUTSIDE;
-      if (v <= -2 && faces.kind[-2 - v] != FACE_NOSLIP) flags |= BF_WALL;
+      if (v <= -2 && faces && faces->kind[-2 - v] != FACE_NOSLIP) flags |= BF_WALL;
       if constexpr (SOLID) {
         const uint64_t m = v >= 0 ? __ldg(solidmask + v) : 0ull;
         s_sm[code] = m;
@@ -886,7 +887,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
   int c0 = NONE;
   if constexpr (XCHG) c0 = __ldg(ex.child0 + b);
   const int flags = stage_block<D, TPB, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, b, t,
-                                               lanes, nbr, solidmask, prm.faces);
+                                               lanes, nbr, solidmask, &prm.faces);
   ParentOut<R> par{nullptr, R(0)};
   if constexpr (XCHG) par = {c0 >= 0 ? s_rc[slot] : nullptr, ex.keep<R>()};
   step_row<D, Q, T, V, SOLID, GHOST_IN, XCHG, false>(gin, gout, b, t, s_nb[slot],

@@ -350,124 +350,169 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
   }
 }
 
-// 128 threads = 128 / 4^D children.  by_parent: child item i is child i % N_c
-// of list[i / N_c] (skipped when the parent has no children, or, in
-// mode_sync, is not refined); else child item i is the block list[i] (a
-// block with a NONE neighbour: the only blocks with interface cells).
-template <int D, int Q, class T, bool SOLID>
-__global__ void __launch_bounds__(128)
-    k_average(const int32_t* __restrict__ list, int64_t n_items, bool by_parent,
-              T* __restrict__ fpar, const T* __restrict__ fch, const int32_t* __restrict__ child0, const int32_t* __restrict__ parent,
-              const uint64_t* __restrict__ cellmask, const int32_t* __restrict__ status,
-              const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
-              double ratio, int mode_sync) {
-  using R = typename Store<T>::R;
-  constexpr int M = Block<D>::M;
-  constexpr int NC = Block<D>::NC;
-  constexpr int NK = Nbr<D>::K;
-  constexpr int CPC = 128 / M;
-  __shared__ R sR[CPC][Q][M];
-  __shared__ int32_t s_row[CPC][2][NK];   // the child's row and its parent's
-  const int slot = threadIdx.x / M;
-  const int l = threadIdx.x - slot * M;
-  const int64_t item = (int64_t)blockIdx.x * CPC + slot;
-  bool valid = item < n_items;
-  int P = 0, c = 0, ch = 0;
-  if (valid) {
-    if (by_parent) {
-      P = list[item / NC];
-      c = (int)(item % NC);
-      const int c0 = child0[P];
-      valid = c0 >= 0 && !(mode_sync && status[P] < ST_REFINED);
-      ch = c0 + c;
-    } else {
-      ch = list[item];
-      P = parent[ch];
-      c = ch - child0[P];
-    }
-  }
-  stage_row<D>(s_row[slot][0], nbr, valid ? ch : NONE, l, M);
-  stage_row<D>(s_row[slot][1], nbr, valid ? P : NONE, l, M);
-  __syncthreads();
-  average_child<D, Q, T, SOLID>(sR[slot], valid, P, c, ch, l, fpar, fch, cellmask, s_row[slot][0], s_row[slot][1], solidmask, ratio,
-                                mode_sync);
+// CTAs of THREADS threads per SM the averaging's register budget is set for.
+template <int Q, class T, int THREADS>
+constexpr int average_min_ctas() {
+  return (Q == 9 ? 1024 : (sizeof(T) == 8 ? 384 : (Q == 27 ? 512 : 768))) / THREADS;
 }
 
-// The level step's averaging (mode 0) over a list of (child block, group)
-// items, the groups of 2^D interface cells of the fine level's boundary
-// blocks whose parent cell is fluid.  One lane per fine cell gathers and
-// rescales it (f_eq + (f - f_eq) r, Section 3.4.3); the 2^D lanes of a group
-// sum their values with a butterfly that halves the directions each lane
-// carries at every exchange (a reduce-scatter: afterwards each lane holds the
-// sums of ceil(Q / 2^D) directions), and each lane stores the means of its
-// directions into the parent cell's slots.  No shared memory, no barrier,
-// every lane busy.
-template <int D, int Q, class T, bool SOLID>
-__global__ void __launch_bounds__(128, 8)
-    k_average_groups(const int32_t* __restrict__ items, int n, T* __restrict__ fpar,
-                     const T* __restrict__ fch, const int32_t* __restrict__ child0,
-                     const int32_t* __restrict__ parent, const int32_t* __restrict__ nbr,
-                     const uint64_t* __restrict__ solidmask, double ratio) {
+// The averaging of a child's cells by x-pairs (3D; by cells in 2D): each of
+// the four lanes of a group holds V of its 2^D cells, gathers and rescales
+// them (f_eq + (f - f_eq) r = f + (f_eq - f)(1 - r), Section 3.4.3), sums them, and
+// the lanes XA and XB apart sum theirs with a reduce-scatter: at each
+// exchange a lane keeps half of the directions it carries, so that afterwards
+// it holds the sums of a quarter of them, whose means it stores into the
+// parent cell's slots.  Every lane of the warp takes part in the exchanges;
+// `take` is the same for the lanes of a group.  Values stay as stored (the
+// shift of the 16-bit types is the same on both sides of a mean).
+template <int D, int Q, class T, int V, bool SOLID, int XA, int XB>
+__device__ __forceinline__ void average_lanes(bool take, int ch, int P, int c, int g,
+                                              const RowPos<D, V>& pos, const int32_t* nb,
+                                              const uint64_t* sm, int flags,
+                                              const T* __restrict__ fch, T* __restrict__ fpar,
+                                              const int32_t* __restrict__ prow,
+                                              const uint64_t* __restrict__ solidmask,
+                                              typename Store<T>::R keep) {
   using S = Store<T>;
   using R = typename S::R;
-  constexpr int NC = Block<D>::NC;            // lanes of a group
-  constexpr int PER = (Q + NC - 1) / NC;      // directions a lane keeps
-  constexpr int QP = PER * NC;
-  const int s = threadIdx.x & (NC - 1);
-  const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / NC;
-  const bool valid = item < n;                // the same for the lanes of a group
-  int ch = 0, g = 0, P = 0, c = 0;
-  if (valid) {
-    const int it = __ldg(items + item);
-    ch = it >> 3;
-    g = it & 7;
-    P = __ldg(parent + ch);
-    c = ch - __ldg(child0 + P);
-  }
-  const int l = Block<D>::cell(2 * (g & 1) + (s & 1), 2 * ((g >> 1) & 1) + ((s >> 1) & 1),
-                               2 * ((g >> 2) & 1) + ((s >> 2) & 1));
+  constexpr int PER = (Q + 3) / 4;      // directions a lane keeps
+  constexpr int QP = 4 * PER;
   R v[QP];
 #pragma unroll
-  for (int p = 0; p < QP; ++p) v[p] = R(0);
-  if (valid) {
-    R f[Q];
-    gather_cell<D, Q, T, SOLID>(f, fch, ch, l, nbr + (size_t)ch * NBR_STRIDE, solidmask);
-    R rho, ux, uy, uz;
-    moments<D, Q>(f, rho, ux, uy, uz);
-    const R usq15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
-    const R r = R(ratio);
-    static_for<0, Q>([&](auto Pp) {
-      const R e = feq<D, Q, Pp>(rho, ux, uy, uz, usq15);
-      v[Pp] = e + (f[Pp] - e) * r;
+  for (int p = Q; p < QP; ++p) v[p] = R(0);
+  if (take) {
+    Vec<T, V> in[Q];
+    gather_row<D, Q, T, V, true, SOLID, false>(in, fch, ch, pos, nb, sm,
+                                               SOLID && (flags & BF_SOLID));
+    static_for<0, V>([&](auto I) {
+      R f[Q];
+      static_for<0, Q>([&](auto Pp) { f[Pp] = S::raw(in[Pp].v[I]); });
+      const Relax<D, Q, S::kShifted, R> r(f);
+      r.each(f, [&](auto Pp, R d) {
+        const R x = fma_(keep, d, f[Pp]);
+        if constexpr (I == 0) v[Pp] = x;
+        else v[Pp] += x;
+      });
     });
-  }
-  // reduce-scatter over the group: at the exchange with lane s ^ m, the lane
-  // with bit m set keeps the upper half of its K directions, the other the
-  // lower half, each adding the partner's copy of the half it keeps
-  int base = 0;
+  } else {
 #pragma unroll
-  for (int m = NC / 2, K = QP; m >= 1; m >>= 1, K >>= 1) {
-    const bool hi = (s & m) != 0;
+    for (int p = 0; p < Q; ++p) v[p] = R(0);
+  }
+  int base = 0;
+  auto halve = [&](auto K, int x) {     // K directions -> K / 2, with the lane x apart
+    const bool hi = (threadIdx.x & x) != 0;
     if (hi) base += K / 2;
 #pragma unroll
     for (int i = 0; i < K / 2; ++i) {
       const R send = hi ? v[i] : v[i + K / 2];
-      const R recv = __shfl_xor_sync(0xffffffffu, send, m);
+      const R recv = __shfl_xor_sync(0xffffffffu, send, x);
       v[i] = (hi ? v[i + K / 2] : v[i]) + recv;
     }
-  }
-  if (!valid) return;
+  };
+  halve(std::integral_constant<int, QP>{}, XA);
+  halve(std::integral_constant<int, QP / 2>{}, XB);
+  if (!take) return;
   const int pc = Block<D>::cell(2 * (c & 1) + (g & 1), 2 * ((c >> 1) & 1) + ((g >> 1) & 1),
                                 2 * ((c >> 2) & 1) + ((g >> 2) & 1));
-  const int32_t* prow = nbr + (size_t)P * NBR_STRIDE;
-  const R inv = R(1) / R(NC);
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
     const int p = base + j;
     if (p < Q)
       fpar[src_slot<D, Q>(p, P, pc, prow, SOLID ? solidmask : nullptr)] =
-          save_rt<D, Q, T>(v[j] * inv, p);
+          S::from_raw(v[j] * (R(1) / R(Block<D>::NC)));
   }
+}
+
+// Whole children: one warp per child in 3D, two children per warp in 2D (115
+// us per level of the synchronisation of a 256,000-block cavity, D3Q19 FP32;
+// 206 with a thread per cell over the children of every block of the level).
+// by_parent: child item i is child i % N_c of list[i / N_c]; else it is the
+// block list[i].  mode_sync as in average_group_taken.
+template <int D, int Q, class T, bool SOLID>
+__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
+    k_average(const int32_t* __restrict__ list, int64_t n_items, bool by_parent,
+              T* __restrict__ fpar, const T* __restrict__ fch, const int32_t* __restrict__ child0,
+              const int32_t* __restrict__ parent, const uint64_t* __restrict__ cellmask,
+              const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
+              typename Store<T>::R keep, int mode_sync) {
+  constexpr int V = D == 3 ? 2 : 1;
+  constexpr int TPB = Block<D>::M / V;
+  constexpr int NC = Block<D>::NC;
+  constexpr int CPC = 128 / TPB;
+  constexpr int NCODE = D == 2 ? 9 : 27;
+  __shared__ int32_t s_nb[CPC][NCODE];
+  __shared__ uint64_t s_sm[SOLID ? CPC : 1][SOLID ? NCODE : 1];
+  const int slot = threadIdx.x / TPB, t = threadIdx.x % TPB;
+  const int64_t item = (int64_t)blockIdx.x * CPC + slot;
+  const bool valid = item < n_items;
+  int P = 0, c = 0, ch = 0, flags = 0;
+  bool take = false;
+  const RowPos<D, V> pos(t);
+  const int g = (pos.i0 >> 1) + 2 * (Block<D>::cj(pos.l0) >> 1) +
+                (D == 3 ? 4 * (Block<D>::ck(pos.l0) >> 1) : 0);
+  if (valid) {
+    if (by_parent) {
+      P = __ldg(list + item / NC);
+      c = (int)(item % NC);
+      ch = __ldg(child0 + P) + c;
+    } else {
+      ch = __ldg(list + item);
+      P = __ldg(parent + ch);
+      c = ch - __ldg(child0 + P);
+    }
+    take = average_group_taken<D>(cellmask, ch, g, mode_sync);
+    if (SOLID && take) {
+      const int pc = Block<D>::cell(2 * (c & 1) + (g & 1), 2 * ((c >> 1) & 1) + ((g >> 1) & 1),
+                                    2 * ((c >> 2) & 1) + ((g >> 2) & 1));
+      take = !((__ldg(solidmask + P) >> pc) & 1ull);
+    }
+    flags = stage_block<D, TPB, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, ch, t,
+                                       block_lanes<TPB>(), nbr, solidmask, nullptr);
+  }
+  average_lanes<D, Q, T, V, SOLID, (D == 3 ? 2 : 1), (D == 3 ? 8 : 4)>(
+      take, ch, P, c, g, pos, s_nb[slot], SOLID ? s_sm[slot] : nullptr, flags, fch, fpar,
+      nbr + (size_t)P * NBR_STRIDE, solidmask, keep);
+}
+
+// The level step's averaging (mode 0) over a list of (child block, group)
+// items, the groups of 2^D interface cells of the fine level's boundary
+// blocks whose parent cell is fluid: four lanes per group, so every lane is
+// busy.  The kernel is bound by its chain of loads (item, neighbour row,
+// populations, parent's row) and by the sectors its groups half use (64^3
+// cavity with three extra levels: 41 us per launch against 44 with a lane per
+// cell; the FP64 2D cavity, where the lanes' work counts, 1.66 -> 1.57 ms per
+// 20 coarse steps).  Children are groups of N_c IDs from first_child on.
+template <int D, int Q, class T, bool SOLID>
+__global__ void __launch_bounds__(64, (average_min_ctas<Q, T, 64>()))
+    k_average_groups(const int32_t* __restrict__ items, int n, T* __restrict__ fpar,
+                     const T* __restrict__ fch, int first_child,
+                     const int32_t* __restrict__ parent, const int32_t* __restrict__ nbr,
+                     const uint64_t* __restrict__ solidmask, typename Store<T>::R keep) {
+  constexpr int V = D == 3 ? 2 : 1;
+  constexpr int NC = Block<D>::NC;
+  constexpr int NCODE = D == 2 ? 9 : 27;
+  constexpr int GPC = 64 / 4;
+  __shared__ int32_t s_nb[GPC][NCODE];
+  __shared__ uint64_t s_sm[SOLID ? GPC : 1][SOLID ? NCODE : 1];
+  const int slot = threadIdx.x / 4, s = threadIdx.x & 3;
+  const int64_t item = (int64_t)blockIdx.x * GPC + slot;
+  const bool valid = item < n;
+  int ch = first_child, g = 0, P = 0, flags = 0;
+  if (valid) {
+    const int it = __ldg(items + item);
+    ch = it >> 3;
+    g = it & 7;
+    P = __ldg(parent + ch);
+    flags = stage_block<D, 4, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, ch, s,
+                                     block_lanes<4>(), nbr, solidmask, nullptr);
+  }
+  const int l = D == 3 ? Block<D>::cell(2 * (g & 1), 2 * ((g >> 1) & 1) + (s & 1),
+                                        2 * ((g >> 2) & 1) + (s >> 1))
+                       : Block<D>::cell(2 * (g & 1) + (s & 1), 2 * ((g >> 1) & 1) + (s >> 1), 0);
+  const RowPos<D, V> pos(l / V);
+  average_lanes<D, Q, T, V, SOLID, 1, 2>(valid, ch, P, (ch - first_child) & (NC - 1), g, pos,
+                                         s_nb[slot], SOLID ? s_sm[slot] : nullptr, flags, fch, fpar,
+                                         nbr + (size_t)P * NBR_STRIDE, solidmask, keep);
 }
 
 // ================================================ batched instances (lock-step)
@@ -491,7 +536,7 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
   const InstDesc& d = descs[it >> BATCH_SHIFT];
   const int b = (int)(it & BATCH_MASK);
   const int flags = stage_block<D, TPB, false>(s_nb[slot], nullptr, b, t, block_lanes<TPB>(),
-                                               d.nbr, nullptr, d.faces);
+                                               d.nbr, nullptr, &d.faces);
   step_row<D, Q, T, V, false, false, false, false>(
       (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[slot], nullptr, flags, 0ull,
       R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
@@ -603,7 +648,7 @@ __device__ __forceinline__ void persist_collide(const InstDesc& d, const uint32_
   for (int s = threadIdx.x / TPB; s < nblk; s += THREADS / TPB) {
     const int b = (int)(__ldg(items + s) & BATCH_MASK);
     const int flags = stage_block<D, TPB, false>(s_nb[s], nullptr, b, t, block_lanes<TPB>(),
-                                                 d.nbr, nullptr, d.faces);
+                                                 d.nbr, nullptr, &d.faces);
     step_row<D, Q, T, V, false, false, false, true>(
         (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[s], nullptr, flags, 0ull,
         R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
@@ -1291,20 +1336,23 @@ struct Launch {
   }
   static void average(cudaStream_t s, const int32_t* list, int n, bool by_parent, void* fpar,
                       const void* fch, const int32_t* child0,
-                      const int32_t* parent, const uint64_t* nm, const int32_t* status,
+                      const int32_t* parent, const uint64_t* nm,
                       const int32_t* nbr, const uint64_t* sm, double ratio, int mode_sync,
                       bool solid) {
     if (n <= 0) return;
+    constexpr int CPC = 128 / (M / (D == 3 ? 2 : 1));
     const int64_t items = by_parent ? (int64_t)n * Block<D>::NC : (int64_t)n;
-    const int grid = (int)((items + 128 / M - 1) / (128 / M));
+    const int grid = (int)((items + CPC - 1) / CPC);
+    using R = typename Store<T>::R;
+    const R keep = R(1.0 - ratio);
     if (solid)
       k_average<D, Q, T, true><<<grid, 128, 0, s>>>(list, items, by_parent, (T*)fpar,
-                                                   (const T*)fch, child0, parent, nm,
-                                                   status, nbr, sm, ratio, mode_sync);
+                                                   (const T*)fch, child0, parent, nm, nbr, sm,
+                                                   keep, mode_sync);
     else
       k_average<D, Q, T, false><<<grid, 128, 0, s>>>(list, items, by_parent, (T*)fpar,
-                                                    (const T*)fch, child0, parent, nm,
-                                                    status, nbr, nullptr, ratio, mode_sync);
+                                                    (const T*)fch, child0, parent, nm, nbr,
+                                                    nullptr, keep, mode_sync);
   }
   static void criterion(cudaStream_t s, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* sm, const int32_t* status, int level,
                         int lmax, double inv_dx, int ns, int ni, int8_t* marks, double* w2out) {
@@ -1402,19 +1450,19 @@ struct Launch {
   }
 
   static void average_groups(cudaStream_t s, const int32_t* items, int n, void* fpar,
-                             const void* fch, const int32_t* child0,
+                             const void* fch, int64_t first_child,
                              const int32_t* parent, const int32_t* nbr, const uint64_t* sm,
                              double ratio, bool solid) {
     if (n <= 0) return;
-    const int grid = (int)(((int64_t)n * Block<D>::NC + 127) / 128);
+    const int grid = grid_for((int64_t)n, 16);
+    using R = typename Store<T>::R;
+    const R keep = R(1.0 - ratio);
     if (solid)
-      k_average_groups<D, Q, T, true><<<grid, 128, 0, s>>>(items, n, (T*)fpar, (const T*)fch,
-                                                           child0, parent, nbr, sm,
-                                                           ratio);
+      k_average_groups<D, Q, T, true><<<grid, 64, 0, s>>>(
+          items, n, (T*)fpar, (const T*)fch, (int)first_child, parent, nbr, sm, keep);
     else
-      k_average_groups<D, Q, T, false><<<grid, 128, 0, s>>>(items, n, (T*)fpar, (const T*)fch,
-                                                            child0, parent, nbr,
-                                                            nullptr, ratio);
+      k_average_groups<D, Q, T, false><<<grid, 64, 0, s>>>(
+          items, n, (T*)fpar, (const T*)fch, (int)first_child, parent, nbr, nullptr, keep);
   }
 
   template <int THREADS>
