@@ -85,33 +85,6 @@ template <int D> struct Block {
   }
 };
 
-// Chebyshev distance (cells) from cell (i,j,k) to the nearest block region in
-// a direction flagged in `none_mask` (bit k set when nbr[k] == NONE); 0 when
-// no bit is set.  Class: d in {1,2} ghost, {3,4} interface, else interior
-// (Section 3.4).
-template <int D>
-__device__ __forceinline__ int cell_class(uint32_t none_mask, int i, int j, int k) {
-  using NV = typename Nbr<D>::V;
-  int best = 99;
-  uint32_t m = none_mask & ~1u;
-  while (m) {
-    int d = __ffs(m) - 1;
-    m &= m - 1;
-    int sx = 0, sy = 0, sz = 0;
-    // direction vectors of the neighbour numbering
-    static_for<1, Nbr<D>::K>([&](auto P) {
-      constexpr int vx = NV::cx[P], vy = NV::cy[P], vz = NV::cz[P];
-      if (P == d) { sx = vx; sy = vy; sz = vz; }
-    });
-    int dist = 0;
-    dist = max(dist, sx < 0 ? i + 1 : (sx > 0 ? 4 - i : 0));
-    dist = max(dist, sy < 0 ? j + 1 : (sy > 0 ? 4 - j : 0));
-    if (D == 3) dist = max(dist, sz < 0 ? k + 1 : (sz > 0 ? 4 - k : 0));
-    best = min(best, dist);
-  }
-  return best <= 2 ? 2 : (best <= 4 ? 1 : 0);   // GHOST, INTERFACE, INTERIOR
-}
-
 // ---------------------------------------------------------- storage traits
 // Values are stored either as the population itself (FP64, FP32) or as the
 // shifted value f - w_p in BF16 / FP16, rounded to nearest even.
