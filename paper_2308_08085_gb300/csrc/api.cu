@@ -837,21 +837,25 @@ int64_t amr_fields(amr_t* h, int what, void* dst, size_t dst_bytes, int dst_on_d
                                          a->nbr, a->sm(), a->red);
       k_sum_partials<<<1, 256, 0, s>>>(g, 4, a->red, out_dev);
     } else {
-      AMR_CUDA(cudaMemsetAsync(out_dev + 4, 0, 3 * 8, s));
-      double* acc = out_dev + 8;
-      AMR_CUDA(cudaMemsetAsync(acc, 0, 3 * 8, s));
-      std::vector<double> tot(3, 0.0), part(3);
+      // each level's sum in a place of its own, read back together
+      double* per_level = out_dev + 8;
+      std::vector<double> part(3 * AMR_MAX_LEVELS, 0.0), tot(3, 0.0);
+      bool any = false;
+      AMR_CUDA(cudaMemsetAsync(per_level, 0, part.size() * 8, s));
       for (int L = 0; L < a->lmax; ++L) {
         if (a->n_active[L] == 0 || !a->solid) continue;
         const double dx = a->cfg.length_x / (a->cfg.nx * std::ldexp(1.0, L));
         const int g = a->ops->force_partial(s, a->active + (size_t)L * cap, (int)a->n_active[L],
                                             a->fbuf(L, 0), a->nbr, a->status,
                                             a->solidmask, 1.0 / a->tau[L], dx, a->red);
-        k_sum_partials<<<1, 256, 0, s>>>(g, 3, a->red, out_dev + 4);
-        AMR_CUDA(cudaMemcpyAsync(part.data(), out_dev + 4, 24, cudaMemcpyDeviceToHost, s));
-        AMR_CUDA(cudaStreamSynchronize(s));
-        for (int v = 0; v < 3; ++v) tot[v] += part[v];
+        k_sum_partials<<<1, 256, 0, s>>>(g, 3, a->red, per_level + 3 * L);
+        any = true;
       }
+      if (any) {
+        AMR_CUDA(cudaMemcpyAsync(part.data(), per_level, part.size() * 8, cudaMemcpyDeviceToHost, s));
+        AMR_CUDA(cudaStreamSynchronize(s));
+      }
+      for (size_t i = 0; i < part.size(); ++i) tot[i % 3] += part[i];
       AMR_CUDA(cudaMemcpyAsync(out_dev, tot.data(), 24, cudaMemcpyHostToDevice, s));
     }
     AMR_CUDA(cudaGetLastError());
