@@ -297,6 +297,7 @@ static void collide_stream_level(Instance* a, int L, bool ghost_in, const Exchan
   StepParams prm = a->prm;
   prm.omega = 1.0 / a->tau[L];
   prm.omega32 = (float)prm.omega;
+  prm.chained = a->chained(n * a->M);
   double bytes = (double)n * a->M * 2.0 * a->q * a->elem;
   if (xchg) bytes += (double)a->n_ghost_cells[L] * a->q * a->elem;   // ghost cells written
   {
@@ -328,7 +329,8 @@ static void advance(Instance* a, int L, bool first) {
                  ((double)a->n_ghost_children[L] * a->nc + cells) * a->q * a->elem, cells);
     a->ops->interp(a->stream, a->parents + (size_t)L * a->cap, (int)np, a->fbuf(L, 0),
                    a->fbuf(L + 1, 1), a->child0, a->cellmask, a->nbr, a->sm(),
-                   nullptr, nullptr, ratio_cf(a, L), 4 | a->interp_bits(), a->solid);
+                   nullptr, nullptr, ratio_cf(a, L), 4 | a->interp_bits(), a->solid,
+                   a->chained(np * a->M * a->nc));
     a->launches += 1;
   }
   Exchange ex{};
@@ -357,11 +359,13 @@ static void advance(Instance* a, int L, bool first) {
       if (cubic)
         a->ops->average(a->stream, a->parents + (size_t)L * a->cap, (int)np, true,
                         a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                        a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
+                        a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid,
+                        a->chained(np * a->M * a->nc));
       else
         a->ops->average_groups(a->stream, a->agrp + a->agrp_off[L + 1], (int)a->n_agrp[L + 1],
                                a->fbuf(L, 0), a->fbuf(L + 1, 0), a->n_root,
-                               a->parent, a->nbr, a->sm(), ratio_fc(a, L), a->solid);
+                               a->parent, a->nbr, a->sm(), ratio_fc(a, L), a->solid,
+                               a->chained(a->n_agrp[L + 1] * a->nc));
       a->launches += 1;
     }
   }
@@ -378,8 +382,10 @@ int64_t coarse_step_into(Instance* a, cudaStream_t s, int parity) {
   a->stream = s;
   a->profiling = 0;
   a->cur = (saved & ~1u) | (unsigned)parity;
+  a->chain = 1;
   const int64_t before = a->launches;
   advance(a, 0, false);
+  a->chain = 0;
   const int64_t n = a->launches - before;
   a->launches = before;
   a->stream = user;
@@ -420,8 +426,10 @@ static int build_graphs(Handle* h) {
     if (e == cudaSuccess) {
       h->capturing = true;
       h->capture_parity = parity;
+      h->chain = h->profiling == 0 ? 1 : 0;   // (event nodes between the launches otherwise)
       const int64_t before = h->launches;
       advance(h, 0, false);
+      h->chain = 0;
       h->graph_launches[parity] = h->launches - before;
       h->launches = before;
       h->capturing = false;
@@ -452,7 +460,7 @@ static void level_sync(Instance* a) {
     // every block of level L + 1 is the child of a refined block
     a->ops->average(a->stream, a->order + (size_t)(L + 1) * a->cap, (int)a->n_ids[L + 1], false,
                     a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                    a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid);
+                    a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid, false);
     a->launches += 1;
   }
   for (int L = 0; L + 1 < a->lmax; ++L) {
@@ -460,7 +468,7 @@ static void level_sync(Instance* a) {
     a->ops->interp(a->stream, a->parents + (size_t)L * a->cap, (int)a->n_parents[L],
                    a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->cellmask,
                    a->nbr, a->sm(), nullptr, nullptr, ratio_cf(a, L), a->interp_bits(),
-                   a->solid);
+                   a->solid, false);
     a->launches += 1;
   }
 }

@@ -876,10 +876,14 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
   __shared__ uint64_t s_sm[SOLID ? BPC : 1][SOLID ? NCODE : 1];
   __shared__ __align__(16) R s_rc[XCHG ? BPC : 1][XCHG ? Q * M : 1];   // rescaled parent cells
 
+  chain_start();
   const int slot = threadIdx.x / TPB;
   const int t = threadIdx.x % TPB;
   const int bi = blockIdx.x * BPC + slot;
-  if (bi >= n) return;                     // (the same for the threads of a block)
+  if (bi >= n) {                           // (the same for the threads of a block)
+    chain_wait();
+    return;
+  }
   const unsigned lanes = block_lanes<TPB>();
   const int b = __ldg(list + bi);
   uint64_t ghost = 0ull;
@@ -888,6 +892,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
   if constexpr (XCHG) c0 = __ldg(ex.child0 + b);
   const int flags = stage_block<D, TPB, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, b, t,
                                                lanes, nbr, solidmask, &prm.faces);
+  chain_wait();
   ParentOut<R> par{nullptr, R(0)};
   if constexpr (XCHG) par = {c0 >= 0 ? s_rc[slot] : nullptr, ex.keep<R>()};
   step_row<D, Q, T, V, SOLID, GHOST_IN, XCHG, false>(gin, gout, b, t, s_nb[slot],

@@ -12,6 +12,23 @@ namespace amr {
 constexpr int NONE = -1;
 constexpr int NBR_STRIDE = 32;   // int32 slots per block row of the nbr table
 
+// ------------------------------------------------- chained kernel launches
+// The launches of a captured coarse step depend on one another in a chain.  A
+// kernel launched as a programmatic dependent starts when every CTA of its
+// predecessor has started; what it reads before chain_wait() is only what no
+// kernel of the step writes (lists, neighbour rows, masks), and chain_wait()
+// returns when the predecessor has finished (which waited for its own).  Both
+// are no-ops in other launches.  A 2D coarse step is 10 to 22 launches of a few
+// microseconds: the start of a launch and its first loads overlap the end of
+// the one before (20 coarse steps of the 128^2 FP32 cavity 1.91 -> 1.61 ms, of
+// the 64^2 FP64 cavity 1.57 -> 1.45).
+__device__ __forceinline__ void chain_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ----------------------------------------------------------- static loops
 template <int B, int E, class F>
 __host__ __device__ __forceinline__ void static_for(F&& f) {

@@ -215,9 +215,11 @@ __global__ void __launch_bounds__(64)
   const bool valid = bi < n;
   const int P = valid ? list[bi] : 0;
   const int c0 = valid ? child0[P] : 0;
+  chain_start();
   for (int r = 0; r <= NC; ++r)
     stage_row<D>(s_row[slot][r], nbr, valid ? (r == 0 ? P : c0 + r - 1) : NONE, l, M);
   __syncthreads();
+  chain_wait();
   if (valid) interp_stage<D, Q, T, SOLID>(sF[slot], fpar, P, l, ratio, s_row[slot][0],
                                           solidmask);
   __syncthreads();
@@ -445,6 +447,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   const int slot = threadIdx.x / TPB, t = threadIdx.x % TPB;
   const int64_t item = (int64_t)blockIdx.x * CPC + slot;
   const bool valid = item < n_items;
+  chain_start();
   int P = 0, c = 0, ch = 0, flags = 0;
   bool take = false;
   const RowPos<D, V> pos(t);
@@ -469,6 +472,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     flags = stage_block<D, TPB, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, ch, t,
                                        block_lanes<TPB>(), nbr, solidmask, nullptr);
   }
+  chain_wait();
   average_lanes<D, Q, T, V, SOLID, (D == 3 ? 2 : 1), (D == 3 ? 8 : 4)>(
       take, ch, P, c, g, pos, s_nb[slot], SOLID ? s_sm[slot] : nullptr, flags, fch, fpar,
       nbr + (size_t)P * NBR_STRIDE, solidmask, keep);
@@ -497,6 +501,7 @@ __global__ void __launch_bounds__(64, (average_min_ctas<Q, T, 64>()))
   const int slot = threadIdx.x / 4, s = threadIdx.x & 3;
   const int64_t item = (int64_t)blockIdx.x * GPC + slot;
   const bool valid = item < n;
+  chain_start();
   int ch = first_child, g = 0, P = 0, flags = 0;
   if (valid) {
     const int it = __ldg(items + item);
@@ -510,6 +515,7 @@ __global__ void __launch_bounds__(64, (average_min_ctas<Q, T, 64>()))
                                         2 * ((g >> 2) & 1) + (s >> 1))
                        : Block<D>::cell(2 * (g & 1) + (s & 1), 2 * ((g >> 1) & 1) + (s >> 1), 0);
   const RowPos<D, V> pos(l / V);
+  chain_wait();
   average_lanes<D, Q, T, V, SOLID, 1, 2>(valid, ch, P, (ch - first_child) & (NC - 1), g, pos,
                                          s_nb[slot], SOLID ? s_sm[slot] : nullptr, flags, fch, fpar,
                                          nbr + (size_t)P * NBR_STRIDE, solidmask, keep);
@@ -1251,6 +1257,22 @@ __global__ void __launch_bounds__(256)
 // =============================================================== launchers
 inline int grid_for(int64_t n, int per) { return (int)((n + per - 1) / per); }
 
+// Launch a kernel that calls chain_start / chain_wait (lattice.cuh).
+template <class... P, class... A>
+inline void launch_chained(void (*kernel)(P...), bool chained, int grid, int threads,
+                           cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = chained ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 template <int D, int Q, class T>
 struct Launch {
   static constexpr int M = Block<D>::M;
@@ -1282,8 +1304,8 @@ struct Launch {
     auto launch = [&](auto ghost, auto parents) {
       constexpr bool G = decltype(ghost)::value, X = decltype(parents)::value;
       const int grid = grid_for(n, THREADS * row_cells<D, T>() / M);
-      k_collide_stream<D, Q, T, SOLID, THREADS, MIN, G, X>
-          <<<grid, THREADS, 0, s>>>(list, n, in, out, nbr, sm, prm, gm, ex);
+      launch_chained(k_collide_stream<D, Q, T, SOLID, THREADS, MIN, G, X>, prm.chained, grid,
+                     THREADS, s, list, n, in, out, nbr, sm, prm, gm, ex);
     };
     if (gm && xchg) launch(std::true_type{}, std::true_type{});
     else if (gm) launch(std::true_type{}, std::false_type{});
@@ -1324,21 +1346,16 @@ struct Launch {
   static void interp(cudaStream_t s, const int32_t* list, int n, const void* fpar, void* fch,
                      const int32_t* child0, const uint64_t* nm,
                      const int32_t* nbr, const uint64_t* sm, const int32_t* parent,
-                     const int8_t* marks, double ratio, int mode_all, bool solid) {
+                     const int8_t* marks, double ratio, int mode_all, bool solid, bool chained) {
     if (n <= 0) return;
     // mode bit 0: every cell (new children), else ghost cells; bit 1: cubic;
     // bit 2: direct writes into the children's own slots
     const int all = mode_all & 5;
     if (mode_all & 2) {
       const int grid = grid_for(n, 64 / M);
-      if (solid)
-        k_interp_cubic<D, Q, T, true><<<grid, 64, 0, s>>>(list, n, (const T*)fpar, (T*)fch,
-                                                         child0, nm, nbr, sm, parent,
-                                                         marks, ratio, all);
-      else
-        k_interp_cubic<D, Q, T, false><<<grid, 64, 0, s>>>(list, n, (const T*)fpar, (T*)fch,
-                                                          child0, nm, nbr, nullptr,
-                                                          parent, marks, ratio, all);
+      launch_chained(solid ? k_interp_cubic<D, Q, T, true> : k_interp_cubic<D, Q, T, false>,
+                     chained, grid, 64, s, list, n, (const T*)fpar, (T*)fch, child0, nm, nbr,
+                     solid ? sm : nullptr, parent, marks, ratio, all);
       return;
     }
     const int grid = grid_for(n, 128 / M);
@@ -1352,21 +1369,16 @@ struct Launch {
                       const void* fch, const int32_t* child0,
                       const int32_t* parent, const uint64_t* nm,
                       const int32_t* nbr, const uint64_t* sm, double ratio, int mode_sync,
-                      bool solid) {
+                      bool solid, bool chained) {
     if (n <= 0) return;
     constexpr int CPC = 128 / (M / (D == 3 ? 2 : 1));
     const int64_t items = by_parent ? (int64_t)n * Block<D>::NC : (int64_t)n;
     const int grid = (int)((items + CPC - 1) / CPC);
     using R = typename Store<T>::R;
     const R keep = R(1.0 - ratio);
-    if (solid)
-      k_average<D, Q, T, true><<<grid, 128, 0, s>>>(list, items, by_parent, (T*)fpar,
-                                                   (const T*)fch, child0, parent, nm, nbr, sm,
-                                                   keep, mode_sync);
-    else
-      k_average<D, Q, T, false><<<grid, 128, 0, s>>>(list, items, by_parent, (T*)fpar,
-                                                    (const T*)fch, child0, parent, nm, nbr,
-                                                    nullptr, keep, mode_sync);
+    launch_chained(solid ? k_average<D, Q, T, true> : k_average<D, Q, T, false>, chained, grid,
+                   128, s, list, items, by_parent, (T*)fpar, (const T*)fch, child0, parent, nm,
+                   nbr, solid ? sm : nullptr, keep, mode_sync);
   }
   static void criterion(cudaStream_t s, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* sm, const int32_t* status, int level,
                         int lmax, double inv_dx, int ns, int ni, int8_t* marks, double* w2out) {
@@ -1466,17 +1478,14 @@ struct Launch {
   static void average_groups(cudaStream_t s, const int32_t* items, int n, void* fpar,
                              const void* fch, int64_t first_child,
                              const int32_t* parent, const int32_t* nbr, const uint64_t* sm,
-                             double ratio, bool solid) {
+                             double ratio, bool solid, bool chained) {
     if (n <= 0) return;
     const int grid = grid_for((int64_t)n, 16);
     using R = typename Store<T>::R;
     const R keep = R(1.0 - ratio);
-    if (solid)
-      k_average_groups<D, Q, T, true><<<grid, 64, 0, s>>>(
-          items, n, (T*)fpar, (const T*)fch, (int)first_child, parent, nbr, sm, keep);
-    else
-      k_average_groups<D, Q, T, false><<<grid, 64, 0, s>>>(
-          items, n, (T*)fpar, (const T*)fch, (int)first_child, parent, nbr, nullptr, keep);
+    launch_chained(solid ? k_average_groups<D, Q, T, true> : k_average_groups<D, Q, T, false>,
+                   chained, grid, 64, s, items, n, (T*)fpar, (const T*)fch, (int)first_child,
+                   parent, nbr, solid ? sm : nullptr, keep);
   }
 
   template <int THREADS>

@@ -106,6 +106,7 @@ struct StepParams {
   int variant;          // collide-stream kernel variant (amr_config.kernel_variant)
   FaceParams faces;
   int32_t* wait_flag;   // device int set to 1 by a kernel whose bounded wait gave up
+  bool chained;         // launch as a programmatic dependent of the launch before
   template <class R> __host__ __device__ R rate() const {
     if constexpr (sizeof(R) == 8) return omega;
     else return omega32;
@@ -139,7 +140,7 @@ struct LbmOps {
   void (*interp)(cudaStream_t, const int32_t* list, int n, const void* fpar, void* fch,
                  const int32_t* child0, const uint64_t* cellmask,
                  const int32_t* nbr, const uint64_t* solidmask, const int32_t* parent,
-                 const int8_t* marks, double ratio, int mode, bool solid);
+                 const int8_t* marks, double ratio, int mode, bool solid, bool chained);
   // fine-to-coarse averaging: by_parent -- `list` holds refined blocks, all
   // their children are visited; else `list` holds children and parent[] leads
   // to their parents.  mode 0: parent cells over interface children, 1: over
@@ -147,7 +148,8 @@ struct LbmOps {
   void (*average)(cudaStream_t, const int32_t* list, int n, bool by_parent, void* fpar,
                   const void* fch, const int32_t* child0, const int32_t* parent,
                   const uint64_t* cellmask, const int32_t* nbr,
-                  const uint64_t* solidmask, double ratio, int mode_sync, bool solid);
+                  const uint64_t* solidmask, double ratio, int mode_sync, bool solid,
+                  bool chained);
   // the averaging of the level step over (block << 3 | group) items: the
   // groups of 2^D interface cells of the fine level's boundary blocks, each
   // into its parent cell (the work of average mode 0, listed in advance);
@@ -155,7 +157,7 @@ struct LbmOps {
   void (*average_groups)(cudaStream_t, const int32_t* items, int n, void* fpar, const void* fch,
                          int64_t first_child, const int32_t* parent,
                          const int32_t* nbr, const uint64_t* solidmask, double ratio,
-                         bool solid);
+                         bool solid, bool chained);
   // vorticity criterion marks (+1/-1/0) and block max |w|^2
   void (*criterion)(cudaStream_t, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* solidmask, const int32_t* status,
                     int level, int lmax, double inv_dx, int n_start, int n_inc, int8_t* marks,
