@@ -610,7 +610,7 @@ __device__ __forceinline__ int stage_block(int32_t* s_nb, uint64_t* s_sm, int b,
       if (v < 0) flags |= BF_OUTSIDE;
       if (v <= -2 && faces && faces->kind[-2 - v] != FACE_NOSLIP) flags |= BF_WALL;
       if constexpr (SOLID) {
-        const uint64_t m = v >= 0 ? __ldg(solidmask + v) : 0ull;
+        const uint64_t m = v >= 0 && solidmask ? __ldg(solidmask + v) : 0ull;
         s_sm[code] = m;
         if (m) flags |= BF_SOLID;
       }

@@ -820,71 +820,123 @@ constexpr size_t persist_smem_bytes() {
          sizeof(int32_t) * (THREADS / Block<D>::M) * (1 + Block<D>::NC) * Nbr<D>::K;
 }
 
+// ================================================ whole blocks, read only
+// The kernels below read the pre-collision populations of whole blocks by
+// x-rows (gather_row): a warp per block in 3D, two blocks per warp in 2D.
+template <int D, class T>
+struct BlockRows {
+  static constexpr int V = D == 3 ? 2 : 1;
+  static constexpr int TPB = Block<D>::M / V;
+  static constexpr int NCODE = D == 2 ? 9 : 27;
+  static constexpr int BPC = 128 / TPB;     // blocks of a CTA of 128 threads
+  struct Shared {
+    int32_t nb[BPC][NCODE];
+    uint64_t sm[BPC][NCODE];
+  };
+};
+
+// Populations of the V cells of this thread of block b (`slot` of its CTA).
+template <int D, int Q, class T>
+__device__ __forceinline__ void read_rows(Vec<T, BlockRows<D, T>::V> (&g)[Q], const T* f, int b,
+                                          int slot, const RowPos<D, BlockRows<D, T>::V>& pos,
+                                          typename BlockRows<D, T>::Shared& s,
+                                          const int32_t* __restrict__ nbr,
+                                          const uint64_t* __restrict__ solidmask) {
+  using B = BlockRows<D, T>;
+  const int flags = stage_block<D, B::TPB, true>(s.nb[slot], s.sm[slot], b, threadIdx.x % B::TPB,
+                                                 block_lanes<B::TPB>(), nbr, solidmask, nullptr);
+  gather_row<D, Q, T, B::V, true, true, false>(g, f, b, pos, s.nb[slot], s.sm[slot],
+                                               flags & BF_SOLID);
+}
+
+// Block-local first-order difference of a value along AXIS (forward, backward
+// at the last cell) for the V cells of a thread; val: the thread's values.
+template <int D, int V, int AXIS, class R>
+__device__ __forceinline__ void block_diff(R (&out)[V], const R (&val)[V],
+                                           const RowPos<D, V>& pos, unsigned lanes) {
+  const int lane = threadIdx.x & 31;
+  if constexpr (AXIS == 0) {
+    if constexpr (V == 2) {
+      const R next = __shfl_sync(lanes, val[0], pos.i0 == 0 ? lane + 1 : lane);
+      out[0] = val[1] - val[0];
+      out[1] = pos.i0 == 0 ? next - val[1] : out[0];
+    } else {
+      const bool last = pos.i0 == 3;
+      const R o = __shfl_sync(lanes, val[0], last ? lane - 1 : lane + 1);
+      out[0] = last ? val[0] - o : o - val[0];
+    }
+  } else {
+    constexpr int STEP = (AXIS == 1 ? 4 : 16) / V;    // lanes between cells along the axis
+    const bool last = (AXIS == 1 ? Block<D>::cj(pos.l0) : Block<D>::ck(pos.l0)) == 3;
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const R o = __shfl_sync(lanes, val[i], last ? lane - STEP : lane + STEP);
+      out[i] = last ? val[i] - o : o - val[i];
+    }
+  }
+}
+
 // ================================================================ criterion
 // Vorticity magnitude from block-local first-order differences (forward, and
 // backward at the last cell), block maximum of |w|^2, desired level of
 // Algorithm 3 (eps < T evaluated as |w|^2 < 4^T), mark: +1 for a leaf with
 // L_des > L, -1 for a REFINED block with L_des <= L.
 template <int D, int Q, class T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     k_criterion(const int32_t* __restrict__ list, int n, const T* __restrict__ f, const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
                 const int32_t* __restrict__ status, int level, int lmax, double inv_dx,
                 int n_start, int n_inc, int8_t* __restrict__ marks, double* __restrict__ w2out) {
   using S = Store<T>;
   using R = typename S::R;
-  constexpr int M = Block<D>::M;
-  constexpr int BPC = 128 / M;
-  __shared__ R su[BPC][3][M];
-  __shared__ R sw[4];
-  const int slot = threadIdx.x / M;
-  const int l = threadIdx.x - slot * M;
-  const int bi = blockIdx.x * BPC + slot;
-  const bool valid = bi < n;
-  int b = 0;
-  if (valid) {
-    b = list[bi];
+  using B = BlockRows<D, T>;
+  constexpr int V = B::V;
+  __shared__ typename B::Shared sh;
+  const int slot = threadIdx.x / B::TPB, t = threadIdx.x % B::TPB;
+  const int bi = blockIdx.x * B::BPC + slot;
+  if (bi >= n) return;                       // (the same for the threads of a block)
+  const unsigned lanes = block_lanes<B::TPB>();
+  const int b = __ldg(list + bi);
+  const RowPos<D, V> pos(t);
+  Vec<T, V> g[Q];
+  read_rows<D, Q, T>(g, f, b, slot, pos, sh, nbr, solidmask);
+  R u[3][V];
+  static_for<0, V>([&](auto I) {
     R fl[Q];
-    gather_cell<D, Q, T, true>(fl, f, b, l, nbr + (size_t)b * NBR_STRIDE, solidmask);
-    R rho, ux, uy, uz;
-    moments<D, Q>(fl, rho, ux, uy, uz);
-    su[slot][0][l] = ux;
-    su[slot][1][l] = uy;
-    su[slot][2][l] = uz;
-  }
-  __syncthreads();
-  R w2 = R(0);
-  if (valid) {
-    const int i = Block<D>::ci(l), j = Block<D>::cj(l), k = Block<D>::ck(l);
-    // d(u_c)/d(axis) in lattice differences
-    auto diff = [&](int comp, int axis) -> R {
-      const int pos = axis == 0 ? i : (axis == 1 ? j : k);
-      const int st = axis == 0 ? 1 : (axis == 1 ? 4 : 16);
-      return pos < 3 ? su[slot][comp][l + st] - su[slot][comp][l]
-                     : su[slot][comp][l] - su[slot][comp][l - st];
-    };
-    const R s = R(inv_dx);
-    if constexpr (D == 2) {
-      const R wz = (diff(1, 0) - diff(0, 1)) * s;
-      w2 = wz * wz;
-    } else {
-      const R wx = (diff(2, 1) - diff(1, 2)) * s;
-      const R wy = (diff(0, 2) - diff(2, 0)) * s;
-      const R wz = (diff(1, 0) - diff(0, 1)) * s;
-      w2 = wx * wx + wy * wy + wz * wz;
+    static_for<0, Q>([&](auto P) { fl[P] = S::template load<D, Q, P>(g[P].v[I]); });
+    R rho;
+    moments<D, Q>(fl, rho, u[0][I], u[1][I], u[2][I]);
+  });
+  const R s = R(inv_dx);
+  R a[V], c[V], w2[V];
+  block_diff<D, V, 0>(a, u[1], pos, lanes);
+  block_diff<D, V, 1>(c, u[0], pos, lanes);
+#pragma unroll
+  for (int i = 0; i < V; ++i) w2[i] = (a[i] - c[i]) * s;
+  if constexpr (D == 2) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) w2[i] = w2[i] * w2[i];
+  } else {
+    R wx[V], wy[V];
+    block_diff<D, V, 1>(a, u[2], pos, lanes);
+    block_diff<D, V, 2>(c, u[1], pos, lanes);
+#pragma unroll
+    for (int i = 0; i < V; ++i) wx[i] = (a[i] - c[i]) * s;
+    block_diff<D, V, 2>(a, u[0], pos, lanes);
+    block_diff<D, V, 0>(c, u[2], pos, lanes);
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      wy[i] = (a[i] - c[i]) * s;
+      w2[i] = wx[i] * wx[i] + wy[i] * wy[i] + w2[i] * w2[i];
     }
   }
-  // block maximum
-  constexpr int START = M < 32 ? M / 2 : 16;
+  R top = w2[0];
 #pragma unroll
-  for (int off = START; off > 0; off >>= 1) w2 = max(w2, __shfl_xor_sync(0xffffffffu, w2, off));
-  if constexpr (M > 32) {
-    const int warp = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0) sw[warp] = w2;
-    __syncthreads();
-    w2 = max(sw[2 * slot], sw[2 * slot + 1]);
-  }
-  if (!valid || l != 0) return;
-  const double w2d = (double)w2;
+  for (int i = 1; i < V; ++i) top = max(top, w2[i]);
+#pragma unroll
+  for (int off = B::TPB / 2; off > 0; off >>= 1)
+    top = max(top, __shfl_xor_sync(lanes, top, off));
+  if (t != 0) return;
+  const double w2d = (double)top;
   int ldes = lmax - 1;
   for (int p = 1; p < lmax; ++p) {
     const int T_ = n_start - p * n_inc;
@@ -911,124 +963,148 @@ constexpr int N_FEATURES = 27;
 
 __device__ __forceinline__ float squash(float x) { return copysignf(log1pf(fabsf(x)), x); }
 
+// A warp per block: 14 sums and 13 maxima over its cells by reduce-scatter
+// (16 exchanges each), so that a lane holds one of them and finishes one
+// feature.  (27 threads that each walked the 64 cells in shared memory took 87
+// us per launch on the 90,000 blocks of a cavity.)
 template <int Q, class T>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     k_features(const int32_t* __restrict__ list, int n, const T* __restrict__ f, const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
                int level, int lmax, double inv_dx, float* __restrict__ out) {
   using S = Store<T>;
   using R = typename S::R;
-  constexpr int D = 3, M = 64, BPC = 2, NV = 15;
-  __shared__ float su[BPC][4][M];            // ux, uy, uz, rho
-  __shared__ float sv[BPC][NV][M];           // per-cell values to reduce
-  const int slot = threadIdx.x / M;
-  const int l = threadIdx.x - slot * M;
-  const int bi = blockIdx.x * BPC + slot;
-  const bool valid = bi < n;
-  int b = 0;
-  if (valid) {
-    b = list[bi];
+  using B = BlockRows<3, T>;
+  __shared__ typename B::Shared sh;
+  const int slot = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const int bi = blockIdx.x * B::BPC + slot;
+  if (bi >= n) return;
+  const int b = __ldg(list + bi);
+  const RowPos<3, 2> pos(lane);
+  Vec<T, 2> g[Q];
+  read_rows<3, Q, T>(g, f, b, slot, pos, sh, nbr, solidmask);
+  float u[3][2], rho[2];
+  static_for<0, 2>([&](auto I) {
     R fl[Q];
-    gather_cell<D, Q, T, true>(fl, f, b, l, nbr + (size_t)b * NBR_STRIDE, solidmask);
-    R rho, ux, uy, uz;
-    moments<D, Q>(fl, rho, ux, uy, uz);
-    su[slot][0][l] = (float)ux;
-    su[slot][1][l] = (float)uy;
-    su[slot][2][l] = (float)uz;
-    su[slot][3][l] = (float)rho;
+    static_for<0, Q>([&](auto P) { fl[P] = S::template load<3, Q, P>(g[P].v[I]); });
+    R r, ux, uy, uz;
+    moments<3, Q>(fl, r, ux, uy, uz);
+    rho[I] = (float)r;
+    u[0][I] = (float)ux;
+    u[1][I] = (float)uy;
+    u[2][I] = (float)uz;
+  });
+  const float s = (float)inv_dx;
+  float G[9][2];
+  static_for<0, 3>([&](auto C) {
+    block_diff<3, 2, 0>(G[3 * C], u[C], pos, 0xffffffffu);
+    block_diff<3, 2, 1>(G[3 * C + 1], u[C], pos, 0xffffffffu);
+    block_diff<3, 2, 2>(G[3 * C + 2], u[C], pos, 0xffffffffu);
+  });
+  // sums: 0..8 G, 9 rho, 10..12 u, 13 |w|; maxima: 0..8 |G|, 9 rho, 10 -rho, 11 |u|, 12 |w|
+  float sum[16], top[16];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    G[q][0] *= s;
+    G[q][1] *= s;
+    sum[q] = G[q][0] + G[q][1];
+    top[q] = fmaxf(fabsf(G[q][0]), fabsf(G[q][1]));
   }
-  __syncthreads();
-  if (valid) {
-    const int i = l & 3, j = (l >> 2) & 3, k = l >> 4;
-    const float s = (float)inv_dx;
-    float G[9];
+  float speed[2], om[2];
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int ax = 0; ax < 3; ++ax) {
-        const int pos = ax == 0 ? i : (ax == 1 ? j : k);
-        const int st = ax == 0 ? 1 : (ax == 1 ? 4 : 16);
-        const float d = pos < 3 ? su[slot][c][l + st] - su[slot][c][l]
-                                : su[slot][c][l] - su[slot][c][l - st];
-        G[3 * c + ax] = d * s;
-      }
-    const float wx = G[7] - G[5], wy = G[2] - G[6], wz = G[3] - G[1];
-    const float ux = su[slot][0][l], uy = su[slot][1][l], uz = su[slot][2][l];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) sv[slot][q][l] = G[q];
-    sv[slot][9][l] = su[slot][3][l];
-    sv[slot][10][l] = ux;
-    sv[slot][11][l] = uy;
-    sv[slot][12][l] = uz;
-    sv[slot][13][l] = sqrtf(ux * ux + uy * uy + uz * uz);
-    sv[slot][14][l] = sqrtf(wx * wx + wy * wy + wz * wz);
+  for (int i = 0; i < 2; ++i) {
+    const float wx = G[7][i] - G[5][i], wy = G[2][i] - G[6][i], wz = G[3][i] - G[1][i];
+    speed[i] = sqrtf(u[0][i] * u[0][i] + u[1][i] * u[1][i] + u[2][i] * u[2][i]);
+    om[i] = sqrtf(wx * wx + wy * wy + wz * wz);
   }
-  __syncthreads();
-  if (!valid || l >= N_FEATURES) return;
-  // thread l reduces feature l over the block's 64 cells
-  const int q = l;
-  float acc;
-  if (q < 9) {                                   // mean of G_q
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc += sv[slot][q][c];
-    acc = squash(acc / M);
-  } else if (q < 18) {                           // max |G_q|
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc = fmaxf(acc, fabsf(sv[slot][q - 9][c]));
-    acc = squash(acc);
-  } else if (q == 18) {                          // mean rho
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc += sv[slot][9][c];
-    acc = (acc / M - 1.f) * 100.f;
-  } else if (q == 19) {                          // max - min rho
-    float lo = sv[slot][9][0], hi = lo;
-    for (int c = 1; c < M; ++c) {
-      lo = fminf(lo, sv[slot][9][c]);
-      hi = fmaxf(hi, sv[slot][9][c]);
+  sum[9] = rho[0] + rho[1];
+  sum[10] = u[0][0] + u[0][1];
+  sum[11] = u[1][0] + u[1][1];
+  sum[12] = u[2][0] + u[2][1];
+  sum[13] = om[0] + om[1];
+  sum[14] = sum[15] = 0.f;
+  top[9] = fmaxf(rho[0], rho[1]);
+  top[10] = fmaxf(-rho[0], -rho[1]);
+  top[11] = fmaxf(speed[0], speed[1]);
+  top[12] = fmaxf(om[0], om[1]);
+  top[13] = top[14] = top[15] = 0.f;
+  int q = 0;                                   // the entry this lane ends up with
+#pragma unroll
+  for (int x = 16, K = 16; x >= 2; x >>= 1, K >>= 1) {
+    const bool hi = (lane & x) != 0;
+    if (hi) q += K / 2;
+#pragma unroll
+    for (int i = 0; i < K / 2; ++i) {
+      const float a = hi ? sum[i] : sum[i + K / 2], c = hi ? top[i] : top[i + K / 2];
+      sum[i] = (hi ? sum[i + K / 2] : sum[i]) + __shfl_xor_sync(0xffffffffu, a, x);
+      top[i] = fmaxf(hi ? top[i + K / 2] : top[i], __shfl_xor_sync(0xffffffffu, c, x));
     }
-    acc = (hi - lo) * 100.f;
-  } else if (q < 23) {                           // mean u_x, u_y, u_z
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc += sv[slot][10 + (q - 20)][c];
-    acc = acc / M * 20.f;
-  } else if (q == 23) {                          // max |u|
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc = fmaxf(acc, sv[slot][13][c]);
-    acc *= 20.f;
-  } else if (q == 24) {                          // mean |w|
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc += sv[slot][14][c];
-    acc = squash(acc / M);
-  } else if (q == 25) {                          // max |w|
-    acc = 0.f;
-    for (int c = 0; c < M; ++c) acc = fmaxf(acc, sv[slot][14][c]);
-    acc = squash(acc);
-  } else {                                       // level / L_max
-    acc = (float)level / (float)lmax;
   }
-  out[(size_t)b * N_FEATURES + q] = acc;
+  const float mean = (sum[0] + __shfl_xor_sync(0xffffffffu, sum[0], 1)) / 64.f;
+  const float most = fmaxf(top[0], __shfl_xor_sync(0xffffffffu, top[0], 1));
+  const float minus_min = __shfl_sync(0xffffffffu, most, 20);   // entry 10 (lane bits 16 and 4)
+  float* o = out + (size_t)b * N_FEATURES;
+  if ((lane & 1) == 0) {                       // even lanes finish the sums
+    if (q < 9) o[q] = squash(mean);
+    else if (q == 9) o[18] = (mean - 1.f) * 100.f;
+    else if (q < 13) o[20 + (q - 10)] = mean * 20.f;
+    else if (q == 13) o[24] = squash(mean);
+    else if (q == 14) o[26] = (float)level / (float)lmax;
+  } else {                                     // odd lanes the maxima
+    if (q < 9) o[9 + q] = squash(most);
+    else if (q == 9) o[19] = (most + minus_min) * 100.f;
+    else if (q == 11) o[23] = most * 20.f;
+    else if (q == 12) o[25] = squash(most);
+  }
 }
 
 // ============================================================ exports/imports
+// `wide`: the destination is aligned for vector stores (the caller's pointer
+// need not be).
+template <int V>
+struct Doubles {
+  double v[V];
+};
+template <int V>
+__device__ __forceinline__ void store_doubles(double* at, const Doubles<V>& x, bool wide) {
+  if constexpr (V == 2) {
+    if (wide) {
+      *reinterpret_cast<double2*>(at) = make_double2(x.v[0], x.v[1]);
+      return;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < V; ++c) at[c] = x.v[c];
+}
+
 template <int D, int Q, class T>
-__global__ void k_export_f(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
-                           const T* __restrict__ fb, unsigned cur,
-                           const int32_t* __restrict__ level, const int32_t* __restrict__ nbr,
-                           const uint64_t* __restrict__ solidmask, double* __restrict__ out) {
-  using R = typename Store<T>::R;
-  constexpr int M = Block<D>::M;
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= nb * M) return;
-  const int64_t b = b0 + g / M;
-  const int l = (int)(g % M);
-  const int L = level[b];
+__global__ void __launch_bounds__(128)
+    k_export_f(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
+               const T* __restrict__ fb, unsigned cur, const int32_t* __restrict__ level,
+               const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
+               double* __restrict__ out, bool wide) {
+  using B = BlockRows<D, T>;
+  constexpr int M = Block<D>::M, V = B::V;
+  __shared__ typename B::Shared sh;
+  const int slot = threadIdx.x / B::TPB, t = threadIdx.x % B::TPB;
+  const int64_t i = (int64_t)blockIdx.x * B::BPC + slot;
+  if (i >= nb) return;
+  const int b = (int)(b0 + i);
+  const int L = __ldg(level + b);
+  const RowPos<D, V> pos(t);
+  double* o = out + i * M + pos.l0;
+  const size_t plane = (size_t)nb * M;
   if (L < 0) {
-    for (int p = 0; p < Q; ++p) out[(size_t)p * nb * M + g] = 0.0;
+    for (int p = 0; p < Q; ++p) store_doubles<V>(o + p * plane, Doubles<V>{}, wide);
     return;
   }
-  const T* f = ((cur >> L) & 1u) ? fb : fa;
-  R fl[Q];
-  gather_cell<D, Q, T, true>(fl, f, (int)b, l, nbr + (size_t)b * NBR_STRIDE, solidmask);
-  static_for<0, Q>([&](auto P) { out[(size_t)P * nb * M + g] = (double)fl[P]; });
+  Vec<T, V> g[Q];
+  read_rows<D, Q, T>(g, ((cur >> L) & 1u) ? fb : fa, b, slot, pos, sh, nbr, solidmask);
+  static_for<0, Q>([&](auto P) {
+    Doubles<V> x;
+#pragma unroll
+    for (int c = 0; c < V; ++c) x.v[c] = (double)Store<T>::template load<D, Q, P>(g[P].v[c]);
+    store_doubles<V>(o + P * plane, x, wide);
+  });
 }
 
 template <int D, int Q, class T>
@@ -1051,32 +1127,49 @@ __global__ void k_import_f(int64_t cap, int64_t b0, int64_t nb, T* __restrict__ 
 }
 
 template <int D, int Q, class T>
-__global__ void k_export_rho_u(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
-                               const T* __restrict__ fb, unsigned cur,
-                               const int32_t* __restrict__ level,
-                               const int32_t* __restrict__ nbr,
-                               const uint64_t* __restrict__ solidmask, double* __restrict__ out) {
-  using R = typename Store<T>::R;
-  constexpr int M = Block<D>::M;
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= nb * M) return;
-  const int64_t b = b0 + g / M;
-  const int l = (int)(g % M);
-  const int L = level[b];
-  double* o = out + (size_t)g * (1 + D);
-  if (L < 0) {
-    for (int a = 0; a <= D; ++a) o[a] = 0.0;
-    return;
+__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
+    k_export_rho_u(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
+                   const T* __restrict__ fb, unsigned cur, const int32_t* __restrict__ level,
+                   const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
+                   double* __restrict__ out, bool wide) {
+  using S = Store<T>;
+  using R = typename S::R;
+  using B = BlockRows<D, T>;
+  constexpr int M = Block<D>::M, V = B::V;
+  __shared__ typename B::Shared sh;
+  const int slot = threadIdx.x / B::TPB, t = threadIdx.x % B::TPB;
+  const int64_t i = (int64_t)blockIdx.x * B::BPC + slot;
+  if (i >= nb) return;
+  const int b = (int)(b0 + i);
+  const int L = __ldg(level + b);
+  const RowPos<D, V> pos(t);
+  double v[V][1 + D] = {};
+  if (L >= 0) {
+    Vec<T, V> g[Q];
+    read_rows<D, Q, T>(g, ((cur >> L) & 1u) ? fb : fa, b, slot, pos, sh, nbr, solidmask);
+    static_for<0, V>([&](auto I) {
+      R fl[Q];
+      static_for<0, Q>([&](auto P) { fl[P] = S::template load<D, Q, P>(g[P].v[I]); });
+      R rho, ux, uy, uz;
+      moments<D, Q>(fl, rho, ux, uy, uz);
+      v[I][0] = rho;
+      v[I][1] = ux;
+      v[I][2] = uy;
+      if constexpr (D == 3) v[I][3] = uz;
+    });
   }
-  const T* f = ((cur >> L) & 1u) ? fb : fa;
-  R fl[Q];
-  gather_cell<D, Q, T, true>(fl, f, (int)b, l, nbr + (size_t)b * NBR_STRIDE, solidmask);
-  R rho, ux, uy, uz;
-  moments<D, Q>(fl, rho, ux, uy, uz);
-  o[0] = rho;
-  o[1] = ux;
-  o[2] = uy;
-  if (D == 3) o[3] = uz;
+  double* o = out + (size_t)(i * M + pos.l0) * (1 + D);
+#pragma unroll
+  for (int c = 0; c < V; ++c) {
+    if (D == 3 && wide) {
+      asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(o + 4 * c), "d"(v[c][0]),
+                   "d"(v[c][1]), "d"(v[c][2]), "d"(v[c][D])
+                   : "memory");
+    } else {
+#pragma unroll
+      for (int a = 0; a <= D; ++a) o[(1 + D) * c + a] = v[c][a];
+    }
+  }
 }
 
 // The rest state (f = w_p in every slot; the gather of it is w_p everywhere).
@@ -1383,14 +1476,14 @@ struct Launch {
   static void criterion(cudaStream_t s, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* sm, const int32_t* status, int level,
                         int lmax, double inv_dx, int ns, int ni, int8_t* marks, double* w2out) {
     if (n <= 0) return;
-    k_criterion<D, Q, T><<<grid_for(n, 128 / M), 128, 0, s>>>(
+    k_criterion<D, Q, T><<<grid_for(n, BlockRows<D, T>::BPC), 128, 0, s>>>(
         list, n, (const T*)f, nbr, sm, status, level, lmax, inv_dx, ns, ni, marks, w2out);
   }
   static void export_f(cudaStream_t s, int64_t cap, int64_t b0, int64_t nb, const void* fa,
                        const void* fb, unsigned cur, const int32_t* level, const int32_t* nbr,
                        const uint64_t* sm, double* out) {
-    k_export_f<D, Q, T><<<grid_for(nb * M, 256), 256, 0, s>>>(
-        cap, b0, nb, (const T*)fa, (const T*)fb, cur, level, nbr, sm, out);
+    k_export_f<D, Q, T><<<grid_for(nb, BlockRows<D, T>::BPC), 128, 0, s>>>(
+        cap, b0, nb, (const T*)fa, (const T*)fb, cur, level, nbr, sm, out, (uintptr_t)out % 16 == 0);
   }
   static void import_f(cudaStream_t s, int64_t cap, int64_t b0, int64_t nb, void* fa, void* fb,
                        unsigned cur, const int32_t* level, const int32_t* nbr,
@@ -1401,8 +1494,8 @@ struct Launch {
   static void export_rho_u(cudaStream_t s, int64_t cap, int64_t b0, int64_t nb, const void* fa,
                            const void* fb, unsigned cur, const int32_t* level,
                            const int32_t* nbr, const uint64_t* sm, double* out) {
-    k_export_rho_u<D, Q, T><<<grid_for(nb * M, 256), 256, 0, s>>>(
-        cap, b0, nb, (const T*)fa, (const T*)fb, cur, level, nbr, sm, out);
+    k_export_rho_u<D, Q, T><<<grid_for(nb, BlockRows<D, T>::BPC), 128, 0, s>>>(
+        cap, b0, nb, (const T*)fa, (const T*)fb, cur, level, nbr, sm, out, (uintptr_t)out % 32 == 0);
   }
   static void init_rest(cudaStream_t s, int64_t cap, void* f) {
     k_init_rest<D, Q, T><<<grid_for(cap * M, 256), 256, 0, s>>>(cap, (T*)f);
@@ -1427,7 +1520,7 @@ struct Launch {
                        double inv_dx, float* out) {
     if constexpr (D == 3) {
       if (n > 0)
-        k_features<Q, T><<<grid_for(n, 2), 128, 0, s>>>(list, n, (const T*)f, nbr, sm,
+        k_features<Q, T><<<grid_for(n, 4), 128, 0, s>>>(list, n, (const T*)f, nbr, sm,
                                                         level, lmax, inv_dx, out);
     }
   }
