@@ -233,7 +233,8 @@ __device__ __forceinline__ void scatter_cell(const typename Store<T>::R (&f)[Q],
 // for S': the shift is neither added on load nor removed on store.  One FP64
 // instruction occupies a scheduler for 64 cycles here (32 lanes, measured), so
 // the FP64 kernels are bound by the operations of this function: 4.5 per
-// direction, 7 when each direction is evaluated on its own.
+// direction, 7 when each direction is evaluated on its own.  (-f is an operand
+// modifier; 0 - f would be an operation.)
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float rcp_(float a) { return 1.f / a; }
@@ -331,13 +332,14 @@ struct Relax {
       return uz3;
     }
   }
-  // f_eq - f of every direction (shifted alike), handed to use(p, d)
+  // f_eq of every direction (shifted alike) as a product, handed to use(p, w, x):
+  // f_eq,p = w x, w = w_p rho
   template <class Use>
-  __device__ __forceinline__ void each(const R (&f)[Q], Use&& use) const {
+  __device__ __forceinline__ void each(Use&& use) const {
     using V = VS<D, Q>;
     const R half = R(0.5);
     constexpr double w0 = V::w[0];
-    use(std::integral_constant<int, 0>{}, fma_(R(w0) * rho, base, R(0) - f[0]));
+    use(std::integral_constant<int, 0>{}, R(w0) * rho, base);
     static_for<1, Q>([&](auto P) {
       constexpr int p = P, pb = V::opp[p];
       if constexpr (pb > p) {
@@ -348,12 +350,25 @@ struct Relax {
         const R c = c3<up>();
         const R wr = R(wp) * rho;
         const R S = fma_(half, c * c, base);
-        use(std::integral_constant<int, up>{}, fma_(wr, S + c, R(0) - f[up]));
-        use(std::integral_constant<int, dn>{}, fma_(wr, S - c, R(0) - f[dn]));
+        use(std::integral_constant<int, up>{}, wr, S + c);
+        use(std::integral_constant<int, dn>{}, wr, S - c);
       }
     });
   }
 };
+
+// f + rate (f_eq - f), f_eq = w x.  (Packed pairs have no negated operand; the
+// product form (rate w) x + (1 - rate) f was no faster there: 12.8 against 12.4
+// ms for five coarse steps of the 128x32x32 prism in FP16.)
+__device__ __forceinline__ float relaxed(float f, float w, float x, float rate) {
+  return fmaf(rate, fmaf(w, x, -f), f);
+}
+__device__ __forceinline__ double relaxed(double f, double w, double x, double rate) {
+  return fma(rate, fma(w, x, -f), f);
+}
+__device__ __forceinline__ F2 relaxed(F2 f, F2 w, F2 x, F2 rate) {
+  return fma_(rate, fma_(w, x, F2(0.f) - f), f);
+}
 
 // Value stored in the own slot p of a cell whose link p leaves through wall
 // face `face` (Section 2 boundary equations): the moving-wall bounce-back
@@ -712,12 +727,12 @@ __device__ __forceinline__ void step_row(const T* __restrict__ gin, T* __restric
       else f[P] = S::raw(g[P].v[i]);
     });
     const Relax<D, Q, SH, RW> r(f);
-    r.each(f, [&](auto P, RW d) {
+    r.each([&](auto P, RW w, RW x) {
       if constexpr (XCHG) {
         if (par.rc)
-          *reinterpret_cast<RW*>(par.rc + P * M + pos.l0 + i) = fma_(RW(par.keep), d, f[P]);
+          *reinterpret_cast<RW*>(par.rc + P * M + pos.l0 + i) = relaxed(f[P], w, x, RW(par.keep));
       }
-      f[P] = fma_(RW(om), d, f[P]);
+      f[P] = relaxed(f[P], w, x, RW(om));
     });
     if (flags & BF_WALL) wall_links<D, Q, SH>(f, r, pos.l0 + i, nb, faces);
     static_for<0, Q>([&](auto P) {

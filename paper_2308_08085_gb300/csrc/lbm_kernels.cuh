@@ -390,10 +390,10 @@ __device__ __forceinline__ void average_lanes(bool take, int ch, int P, int c, i
       R f[Q];
       static_for<0, Q>([&](auto Pp) { f[Pp] = S::raw(in[Pp].v[I]); });
       const Relax<D, Q, S::kShifted, R> r(f);
-      r.each(f, [&](auto Pp, R d) {
-        const R x = fma_(keep, d, f[Pp]);
-        if constexpr (I == 0) v[Pp] = x;
-        else v[Pp] += x;
+      r.each([&](auto Pp, R w, R x) {
+        const R y = relaxed(f[Pp], w, x, keep);
+        if constexpr (I == 0) v[Pp] = y;
+        else v[Pp] += y;
       });
     });
   } else {
