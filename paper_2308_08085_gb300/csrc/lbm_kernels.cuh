@@ -190,7 +190,8 @@ constexpr CubicW make_cubic_w() {
 static __constant__ CubicW c_cubic_w = make_cubic_w();
 
 template <int D, int Q, class T, bool SOLID>
-__global__ void __launch_bounds__(64)
+// (ten CTAs per SM: what the shared memory of D3Q27 in FP32 leaves room for)
+__global__ void __launch_bounds__(64, sizeof(typename Store<T>::R) == 8 ? 5 : 10)
     k_interp_cubic(const int32_t* __restrict__ list, int n, const T* __restrict__ fpar,
                    T* __restrict__ fch, const int32_t* __restrict__ child0,
                    const uint64_t* __restrict__ cellmask, const int32_t* __restrict__ nbr,
@@ -352,10 +353,15 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
   }
 }
 
-// CTAs of THREADS threads per SM the averaging's register budget is set for.
+// CTAs of THREADS threads per SM the register budget of the averaging (and of
+// the criterion, the summaries and the export of moments, which hold as much)
+// is set for: 1024 threads for D3Q19 (64 registers), 768 for D3Q27 (80).
+// Measured (marks and summaries of a cavity, D3Q19 / prism with cubic
+// interpolation, D3Q27): 0.91 / 17.8 ms with 768 / 512 threads, 0.88 / 16.9
+// with these, 0.94 / 17.1 with 1152 / 896 (spills).
 template <int Q, class T, int THREADS>
 constexpr int average_min_ctas() {
-  return (Q == 9 ? 1024 : (sizeof(T) == 8 ? 384 : (Q == 27 ? 512 : 768))) / THREADS;
+  return (Q == 9 ? 1024 : (sizeof(T) == 8 ? 384 : (Q == 27 ? 768 : 1024))) / THREADS;
 }
 
 // The averaging of a child's cells by x-pairs (3D; by cells in 2D): each of
