@@ -92,7 +92,8 @@ struct Instance {
   // its predecessor hold the slots its last wave needs less than the next
   // launch gains (64^3 cavity, D3Q19 FP32, 10 coarse steps: 35.5 ms without
   // chaining, 34.9 with this limit, 35.6 with none; prism D3Q27 FP32 cubic:
-  // 17.9 / 17.8 / 26.7; 128^2 FP32 cavity, all launches small: 1.91 -> 1.61).
+  // 17.9 / 17.8 / 26.7 (most of that from its interpolation launches, which
+  // are not chained at all now); 128^2 FP32 cavity, all launches small: 1.91 -> 1.61).
   static constexpr int64_t kChainCells = int64_t(1) << 17;
   int chain = 0;
   bool chained(int64_t cells) {

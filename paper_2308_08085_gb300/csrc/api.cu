@@ -329,8 +329,8 @@ static void advance(Instance* a, int L, bool first) {
                  ((double)a->n_ghost_children[L] * a->nc + cells) * a->q * a->elem, cells);
     a->ops->interp(a->stream, a->parents + (size_t)L * a->cap, (int)np, a->fbuf(L, 0),
                    a->fbuf(L + 1, 1), a->child0, a->cellmask, a->nbr, a->sm(),
-                   nullptr, nullptr, ratio_cf(a, L), 4 | a->interp_bits(), a->solid,
-                   a->chained(np * a->M * a->nc));
+                   nullptr, nullptr, ratio_cf(a, L), 4 | a->interp_bits(), a->solid);
+    a->chained(0);   // (the launch after it may be chained to it)
     a->launches += 1;
   }
   Exchange ex{};
@@ -468,7 +468,7 @@ static void level_sync(Instance* a) {
     a->ops->interp(a->stream, a->parents + (size_t)L * a->cap, (int)a->n_parents[L],
                    a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->cellmask,
                    a->nbr, a->sm(), nullptr, nullptr, ratio_cf(a, L), a->interp_bits(),
-                   a->solid, false);
+                   a->solid);
     a->launches += 1;
   }
 }

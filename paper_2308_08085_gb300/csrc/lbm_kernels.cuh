@@ -220,7 +220,6 @@ __global__ void __launch_bounds__(64, sizeof(typename Store<T>::R) == 8 ? 5 : 10
   for (int r = 0; r <= NC; ++r)
     stage_row<D>(s_row[slot][r], nbr, valid ? (r == 0 ? P : c0 + r - 1) : NONE, l, M);
   __syncthreads();
-  chain_wait();
   if (valid) interp_stage<D, Q, T, SOLID>(sF[slot], fpar, P, l, ratio, s_row[slot][0],
                                           solidmask);
   __syncthreads();
@@ -1445,16 +1444,24 @@ struct Launch {
   static void interp(cudaStream_t s, const int32_t* list, int n, const void* fpar, void* fch,
                      const int32_t* child0, const uint64_t* nm,
                      const int32_t* nbr, const uint64_t* sm, const int32_t* parent,
-                     const int8_t* marks, double ratio, int mode_all, bool solid, bool chained) {
+                     const int8_t* marks, double ratio, int mode_all, bool solid) {
     if (n <= 0) return;
     // mode bit 0: every cell (new children), else ghost cells; bit 1: cubic;
     // bit 2: direct writes into the children's own slots
     const int all = mode_all & 5;
     if (mode_all & 2) {
       const int grid = grid_for(n, 64 / M);
-      launch_chained(solid ? k_interp_cubic<D, Q, T, true> : k_interp_cubic<D, Q, T, false>,
-                     chained, grid, 64, s, list, n, (const T*)fpar, (T*)fch, child0, nm, nbr,
-                     solid ? sm : nullptr, parent, marks, ratio, all);
+      // never a dependent of the launch before: its CTAs would wait with their
+      // shared memory in hand (2D FP64 prism, 4 levels, 8 coarse steps: 4.9 ms
+      // chained, 3.15 not)
+      if (solid)
+        k_interp_cubic<D, Q, T, true><<<grid, 64, 0, s>>>(list, n, (const T*)fpar, (T*)fch,
+                                                         child0, nm, nbr, sm, parent,
+                                                         marks, ratio, all);
+      else
+        k_interp_cubic<D, Q, T, false><<<grid, 64, 0, s>>>(list, n, (const T*)fpar, (T*)fch,
+                                                          child0, nm, nbr, nullptr,
+                                                          parent, marks, ratio, all);
       return;
     }
     const int grid = grid_for(n, 128 / M);

@@ -140,7 +140,7 @@ struct LbmOps {
   void (*interp)(cudaStream_t, const int32_t* list, int n, const void* fpar, void* fch,
                  const int32_t* child0, const uint64_t* cellmask,
                  const int32_t* nbr, const uint64_t* solidmask, const int32_t* parent,
-                 const int8_t* marks, double ratio, int mode, bool solid, bool chained);
+                 const int8_t* marks, double ratio, int mode, bool solid);
   // fine-to-coarse averaging: by_parent -- `list` holds refined blocks, all
   // their children are visited; else `list` holds children and parent[] leads
   // to their parents.  mode 0: parent cells over interface children, 1: over

@@ -889,7 +889,7 @@ static int adapt_t(Instance* a, amr_adapt_stats* st) {
     AMR_CUDA(cudaGetLastError());
     const double ratio = a->tau[L + 1] / (2.0 * a->tau[L]);
     a->ops->interp(s, C + offR[L], (int)nRL[L], a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->cellmask, a->nbr, a->sm(), a->parent, a->marks, ratio,
-                   1 | a->interp_bits(), a->solid, false);
+                   1 | a->interp_bits(), a->solid);
     a->launches += 1;
     AMR_CUDA(cudaGetLastError());
   }
