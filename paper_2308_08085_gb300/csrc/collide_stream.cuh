@@ -94,8 +94,6 @@ constexpr LinkTable<D, Q> make_link_table() {
   return t;
 }
 template <int D, int Q>
-__device__ const LinkTable<D, Q> g_src_geo = make_link_table<D, Q, -1, false>();
-template <int D, int Q>
 __device__ const LinkTable<D, Q> g_tgt_geo = make_link_table<D, Q, +1, false>();
 template <int D, int Q>
 __device__ const LinkTable<D, Q> g_src_k = make_link_table<D, Q, -1, true>();
@@ -285,7 +283,7 @@ struct Relax {
       : rho(rho_), base(base_), ux3(x), uy3(y), uz3(z) {}
   __device__ __forceinline__ explicit Relax(const R (&f)[Q]) {
     using V = VS<D, Q>;
-    // sums of the values, and of the differences along each axis (N[a]: terms so far)
+    // sums of the values, and of the differences along each axis
     R s = f[0], j[3];
     bool any[3] = {false, false, false};
     static_for<1, Q>([&](auto P) {

@@ -151,24 +151,6 @@ template <> struct Store<__half> {
   }
 };
 
-// Runtime-p variants (used off the hot path).
-template <int D, int Q, class T>
-__device__ __forceinline__ typename Store<T>::R load_rt(T v, int p) {
-  typename Store<T>::R r = 0;
-  static_for<0, Q>([&](auto P) {
-    if (P == p) r = Store<T>::template load<D, Q, P>(v);
-  });
-  return r;
-}
-template <int D, int Q, class T>
-__device__ __forceinline__ T save_rt(typename Store<T>::R v, int p) {
-  T r{};
-  static_for<0, Q>([&](auto P) {
-    if (P == p) r = Store<T>::template save<D, Q, P>(v);
-  });
-  return r;
-}
-
 // ------------------------------------------------------- BGK building blocks
 template <int D, int Q, class R>
 __device__ __forceinline__ void moments(const R* f, R& rho, R& ux, R& uy, R& uz) {
