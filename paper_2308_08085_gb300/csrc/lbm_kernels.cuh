@@ -430,9 +430,50 @@ __device__ __forceinline__ void average_lanes(bool take, int ch, int P, int c, i
   }
 }
 
-// Whole children: one warp per child in 3D, two children per warp in 2D (115
-// us per level of the synchronisation of a 256,000-block cavity, D3Q19 FP32;
-// 206 with a thread per cell over the children of every block of the level).
+// The weights as a device table (for a runtime p).
+template <int D, int Q>
+struct WeightTable {
+  float w[Q];
+};
+template <int D, int Q>
+constexpr WeightTable<D, Q> make_weight() {
+  WeightTable<D, Q> t{};
+  for (int p = 0; p < Q; ++p) t.w[p] = float(VS<D, Q>::w[p]);
+  return t;
+}
+template <int D, int Q>
+__device__ const WeightTable<D, Q> g_weight = make_weight<D, Q>();
+
+// Two lanes of a group, x apart, hand one another half of the N directions
+// they carry: NIN values of each before, 2 NIN of N / 2 after, in cell order
+// (those of the lane without bit X first).  `base` becomes the first direction
+// this lane keeps.
+template <int N, int NIN, class R>
+__device__ __forceinline__ void gather_half(R (&out)[N / 2][2 * NIN], const R (&in)[N][NIN], int x,
+                                            int& base) {
+  const bool hi = (threadIdx.x & x) != 0;
+  if (hi) base += N / 2;
+#pragma unroll
+  for (int i = 0; i < N / 2; ++i)
+#pragma unroll
+    for (int c = 0; c < NIN; ++c) {
+      const R keep = hi ? in[i + N / 2][c] : in[i][c];
+      const R recv = __shfl_xor_sync(0xffffffffu, hi ? in[i][c] : in[i + N / 2][c], x);
+      out[i][c] = hi ? recv : keep;
+      out[i][NIN + c] = hi ? keep : recv;
+    }
+}
+
+// Whole children: one warp per child in 3D, two children per warp in 2D.  Each
+// of the four lanes of a group gathers V of its 2^D cells and rescales them
+// (f_eq + (f - f_eq) r, Section 3.4.3); the group's lanes then exchange values
+// until each holds all 2^D of a quarter of the directions, adds them in cell
+// order and stores the means.  The order is part of the result: refinement
+// marks are thresholds on values derived from this state, so its last bits
+// must not follow the layout of the lanes (average_lanes, whose sums go by
+// pairs, serves the level step only).  Synchronisation, criterion, summaries
+// and inference of a 90,000-block cavity, D3Q19 FP32: 0.93 ms; 0.88 with sums
+// by pairs here and in k_features, 1.40 with a thread per cell.
 // by_parent: child item i is child i % N_c of list[i / N_c]; else it is the
 // block list[i].  mode_sync as in average_group_taken.
 template <int D, int Q, class T, bool SOLID>
@@ -441,7 +482,9 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
               T* __restrict__ fpar, const T* __restrict__ fch, const int32_t* __restrict__ child0,
               const int32_t* __restrict__ parent, const uint64_t* __restrict__ cellmask,
               const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
-              typename Store<T>::R keep, int mode_sync) {
+              double ratio, int mode_sync) {
+  using S = Store<T>;
+  using R = typename S::R;
   constexpr int V = D == 3 ? 2 : 1;
   constexpr int TPB = Block<D>::M / V;
   constexpr int NC = Block<D>::NC;
@@ -478,9 +521,51 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
                                        block_lanes<TPB>(), nbr, solidmask, nullptr);
   }
   chain_wait();
-  average_lanes<D, Q, T, V, SOLID, (D == 3 ? 2 : 1), (D == 3 ? 8 : 4)>(
-      take, ch, P, c, g, pos, s_nb[slot], SOLID ? s_sm[slot] : nullptr, flags, fch, fpar,
-      nbr + (size_t)P * NBR_STRIDE, solidmask, keep);
+  constexpr int QP = (Q + 3) / 4 * 4;   // directions, a quarter of them per lane
+  R v[QP][V];
+#pragma unroll
+  for (int p = 0; p < QP; ++p)
+#pragma unroll
+    for (int i = 0; i < V; ++i) v[p][i] = R(0);
+  if (take) {
+    Vec<T, V> in[Q];
+    gather_row<D, Q, T, V, true, SOLID, false>(in, fch, ch, pos, s_nb[slot],
+                                               SOLID ? s_sm[slot] : nullptr,
+                                               SOLID && (flags & BF_SOLID));
+    const R r = R(ratio);
+    static_for<0, V>([&](auto I) {
+      R f[Q];
+      static_for<0, Q>([&](auto Pp) { f[Pp] = S::template load<D, Q, Pp>(in[Pp].v[I]); });
+      R rho, ux, uy, uz;
+      moments<D, Q>(f, rho, ux, uy, uz);
+      const R usq15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
+      static_for<0, Q>([&](auto Pp) {
+        const R e = feq<D, Q, Pp>(rho, ux, uy, uz, usq15);
+        v[Pp][I] = e + (f[Pp] - e) * r;
+      });
+    });
+  }
+  int base = 0;
+  R v2[QP / 2][2 * V], v4[QP / 4][4 * V];
+  gather_half<QP, V>(v2, v, D == 3 ? 2 : 1, base);          // the group's y (2D: x) neighbour
+  gather_half<QP / 2, 2 * V>(v4, v2, D == 3 ? 8 : 4, base);   // its z (2D: y) neighbour
+  if (!take) return;
+  const int pc = Block<D>::cell(2 * (c & 1) + (g & 1), 2 * ((c >> 1) & 1) + ((g >> 1) & 1),
+                                2 * ((c >> 2) & 1) + ((g >> 2) & 1));
+  const R inv = R(1) / R(NC);
+#pragma unroll
+  for (int j = 0; j < QP / 4; ++j) {
+    R sum = R(0);
+#pragma unroll
+    for (int i = 0; i < NC; ++i) sum += v4[j][i];
+    const int p = base + j;
+    if (p < Q) {
+      sum *= inv;
+      if constexpr (S::kShifted) sum -= __ldg(&g_weight<D, Q>.w[p]);
+      fpar[src_slot<D, Q>(p, P, pc, nbr + (size_t)P * NBR_STRIDE, SOLID ? solidmask : nullptr)] =
+          S::from_raw(sum);
+    }
+  }
 }
 
 // The level step's averaging (mode 0) over a list of (child block, group)
@@ -968,10 +1053,10 @@ constexpr int N_FEATURES = 27;
 
 __device__ __forceinline__ float squash(float x) { return copysignf(log1pf(fabsf(x)), x); }
 
-// A warp per block: 14 sums and 13 maxima over its cells by reduce-scatter
-// (16 exchanges each), so that a lane holds one of them and finishes one
-// feature.  (27 threads that each walked the 64 cells in shared memory took 87
-// us per launch on the 90,000 blocks of a cavity.)
+// A warp per block: the cells' values go to shared memory, 16 rows of 64, and
+// 16 lanes walk a row each.  The sums are taken in cell order: the proposal
+// compares a function of them with a threshold, so that the marks hang on
+// their last bits.
 template <int Q, class T>
 __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     k_features(const int32_t* __restrict__ list, int n, const T* __restrict__ f, const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
@@ -979,6 +1064,8 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   using S = Store<T>;
   using R = typename S::R;
   using B = BlockRows<3, T>;
+  // (rows of 68 words: 16-byte reads of eight rows touch every bank once)
+  __shared__ __align__(16) float s_row[B::BPC][16][68];
   __shared__ typename B::Shared sh;
   const int slot = threadIdx.x / 32, lane = threadIdx.x & 31;
   const int bi = blockIdx.x * B::BPC + slot;
@@ -1005,60 +1092,63 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     block_diff<3, 2, 1>(G[3 * C + 1], u[C], pos, 0xffffffffu);
     block_diff<3, 2, 2>(G[3 * C + 2], u[C], pos, 0xffffffffu);
   });
-  // sums: 0..8 G, 9 rho, 10..12 u, 13 |w|; maxima: 0..8 |G|, 9 rho, 10 -rho, 11 |u|, 12 |w|
-  float sum[16], top[16];
-#pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    G[q][0] *= s;
-    G[q][1] *= s;
-    sum[q] = G[q][0] + G[q][1];
-    top[q] = fmaxf(fabsf(G[q][0]), fabsf(G[q][1]));
-  }
+  // rows: 0..8 G, 9 rho, 10..12 u, 13 |u|, 14 |w|, 15 -rho
+  float (*row)[68] = s_row[slot];
+  auto put = [&](int q, float a, float c) {
+    *reinterpret_cast<float2*>(&row[q][pos.l0]) = make_float2(a, c);
+  };
   float speed[2], om[2];
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) G[q][i] *= s;
     const float wx = G[7][i] - G[5][i], wy = G[2][i] - G[6][i], wz = G[3][i] - G[1][i];
     speed[i] = sqrtf(u[0][i] * u[0][i] + u[1][i] * u[1][i] + u[2][i] * u[2][i]);
     om[i] = sqrtf(wx * wx + wy * wy + wz * wz);
   }
-  sum[9] = rho[0] + rho[1];
-  sum[10] = u[0][0] + u[0][1];
-  sum[11] = u[1][0] + u[1][1];
-  sum[12] = u[2][0] + u[2][1];
-  sum[13] = om[0] + om[1];
-  sum[14] = sum[15] = 0.f;
-  top[9] = fmaxf(rho[0], rho[1]);
-  top[10] = fmaxf(-rho[0], -rho[1]);
-  top[11] = fmaxf(speed[0], speed[1]);
-  top[12] = fmaxf(om[0], om[1]);
-  top[13] = top[14] = top[15] = 0.f;
-  int q = 0;                                   // the entry this lane ends up with
 #pragma unroll
-  for (int x = 16, K = 16; x >= 2; x >>= 1, K >>= 1) {
-    const bool hi = (lane & x) != 0;
-    if (hi) q += K / 2;
+  for (int q = 0; q < 9; ++q) put(q, G[q][0], G[q][1]);
+  put(9, rho[0], rho[1]);
 #pragma unroll
-    for (int i = 0; i < K / 2; ++i) {
-      const float a = hi ? sum[i] : sum[i + K / 2], c = hi ? top[i] : top[i + K / 2];
-      sum[i] = (hi ? sum[i + K / 2] : sum[i]) + __shfl_xor_sync(0xffffffffu, a, x);
-      top[i] = fmaxf(hi ? top[i + K / 2] : top[i], __shfl_xor_sync(0xffffffffu, c, x));
-    }
+  for (int a = 0; a < 3; ++a) put(10 + a, u[a][0], u[a][1]);
+  put(13, speed[0], speed[1]);
+  put(14, om[0], om[1]);
+  put(15, -rho[0], -rho[1]);
+  __syncwarp();
+  // largest magnitude, of rho and -rho the largest value
+  const int q = lane & 15;
+  const bool is_rho = q == 9 || q == 15;
+  float sum = 0.f, top = is_rho ? row[q][0] : 0.f;
+#pragma unroll 4
+  for (int c = 0; c < 64; c += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(&row[q][c]);
+    sum += x.x;
+    sum += x.y;
+    sum += x.z;
+    sum += x.w;
+    top = fmaxf(top, is_rho ? x.x : fabsf(x.x));
+    top = fmaxf(top, is_rho ? x.y : fabsf(x.y));
+    top = fmaxf(top, is_rho ? x.z : fabsf(x.z));
+    top = fmaxf(top, is_rho ? x.w : fabsf(x.w));
   }
-  const float mean = (sum[0] + __shfl_xor_sync(0xffffffffu, sum[0], 1)) / 64.f;
-  const float most = fmaxf(top[0], __shfl_xor_sync(0xffffffffu, top[0], 1));
-  const float minus_min = __shfl_sync(0xffffffffu, most, 20);   // entry 10 (lane bits 16 and 4)
+  const float minus_min = __shfl_sync(0xffffffffu, top, 15);
+  const float mean = sum / 64.f;
   float* o = out + (size_t)b * N_FEATURES;
-  if ((lane & 1) == 0) {                       // even lanes finish the sums
-    if (q < 9) o[q] = squash(mean);
-    else if (q == 9) o[18] = (mean - 1.f) * 100.f;
-    else if (q < 13) o[20 + (q - 10)] = mean * 20.f;
-    else if (q == 13) o[24] = squash(mean);
-    else if (q == 14) o[26] = (float)level / (float)lmax;
-  } else {                                     // odd lanes the maxima
-    if (q < 9) o[9 + q] = squash(most);
-    else if (q == 9) o[19] = (most + minus_min) * 100.f;
-    else if (q == 11) o[23] = most * 20.f;
-    else if (q == 12) o[25] = squash(most);
+  if (lane < 9) {
+    o[lane] = squash(mean);
+    o[9 + lane] = squash(top);
+  } else if (lane == 9) {
+    o[18] = (mean - 1.f) * 100.f;
+    o[19] = (top + minus_min) * 100.f;
+  } else if (lane < 13) {
+    o[20 + (lane - 10)] = mean * 20.f;
+  } else if (lane == 13) {
+    o[23] = top * 20.f;
+  } else if (lane == 14) {
+    o[24] = squash(mean);
+    o[25] = squash(top);
+  } else if (lane == 15) {
+    o[26] = (float)level / (float)lmax;
   }
 }
 
@@ -1480,11 +1570,9 @@ struct Launch {
     constexpr int CPC = 128 / (M / (D == 3 ? 2 : 1));
     const int64_t items = by_parent ? (int64_t)n * Block<D>::NC : (int64_t)n;
     const int grid = (int)((items + CPC - 1) / CPC);
-    using R = typename Store<T>::R;
-    const R keep = R(1.0 - ratio);
     launch_chained(solid ? k_average<D, Q, T, true> : k_average<D, Q, T, false>, chained, grid,
                    128, s, list, items, by_parent, (T*)fpar, (const T*)fch, child0, parent, nm,
-                   nbr, solid ? sm : nullptr, keep, mode_sync);
+                   nbr, solid ? sm : nullptr, ratio, mode_sync);
   }
   static void criterion(cudaStream_t s, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* sm, const int32_t* status, int level,
                         int lmax, double inv_dx, int ns, int ni, int8_t* marks, double* w2out) {
