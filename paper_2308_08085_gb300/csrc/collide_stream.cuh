@@ -504,7 +504,7 @@ struct RowPos {
 // block's neighbour row in geometric order; `sm` (SOLID) the solid cells of
 // those blocks, read when any_solid.
 template <int D, int Q, class T, int V, bool CHECK, bool SOLID, bool COH>
-__device__ __forceinline__ void gather_row(Vec<T, V> (&g)[Q], const T* __restrict__ gin, int b,
+__device__ __forceinline__ void gather_row(Vec<T, V> (&g)[Q], const T* gin, int b,
                                            const RowPos<D, V>& pos, const int32_t* nb,
                                            const uint64_t* sm, bool any_solid,
                                            const T* in_place = nullptr) {
@@ -684,7 +684,7 @@ struct ParentOut {
 // with its children, and its pre-collision values rescaled to the fine level
 // (f_eq + (f - f_eq) r_cf = f + (f_eq - f)(1 - r_cf), Section 3.4.1) go there.
 template <int D, int Q, class T, int V, bool SOLID, bool GHOST, bool XCHG, bool COH>
-__device__ __forceinline__ void step_row(const T* __restrict__ gin, T* __restrict__ gout, int b,
+__device__ __forceinline__ void step_row(const T* gin, T* gout, int b,
                                          int t, const int32_t* nb, const uint64_t* sm, int flags,
                                          uint64_t ghost, typename Store<T>::R om,
                                          const FaceParams& faces,
@@ -789,7 +789,7 @@ __device__ const CornerWeights<D> g_corner = make_corner_weights<D>();
 template <int D, int Q, class T, int V>
 __device__ __forceinline__ void interp_rows(const typename Store<T>::R* rc, int t, int c0,
                                             const uint64_t* __restrict__ cellmask,
-                                            T* __restrict__ fout,
+                                            T* fout,
                                             const uint64_t* __restrict__ solidmask) {
   using S = Store<T>;
   using R = typename S::R;
@@ -873,8 +873,8 @@ __device__ __forceinline__ void interp_rows(const typename Store<T>::R* rc, int 
 // cells to its children's interpolation, need no CTA barrier.
 template <int D, int Q, class T, bool SOLID, int THREADS, int MIN_CTAS, bool GHOST_IN, bool XCHG>
 __global__ void __launch_bounds__(THREADS, MIN_CTAS)
-    k_collide_stream(const int32_t* __restrict__ list, int n, const T* __restrict__ gin,
-                     T* __restrict__ gout, const int32_t* __restrict__ nbr,
+    k_collide_stream(const int32_t* __restrict__ list, int n, const T* gin,
+                     T* gout, const int32_t* __restrict__ nbr,
                      const uint64_t* __restrict__ solidmask,
                      const __grid_constant__ StepParams prm,
                      const uint64_t* __restrict__ cellmask, const __grid_constant__ Exchange ex) {

@@ -22,6 +22,13 @@ constexpr int NBR_STRIDE = 32;   // int32 slots per block row of the nbr table
 // microseconds: the start of a launch and its first loads overlap the end of
 // the one before (20 coarse steps of the 128^2 FP32 cavity 1.91 -> 1.61 ms, of
 // the 64^2 FP64 cavity 1.57 -> 1.45).
+//
+// A dependent kernel is resident while its predecessor writes populations.
+// `const __restrict__` would promise the compiler that nobody writes them
+// during the kernel: it could read them through the read-only path or move the
+// loads above the wait, which clobbers only memory that others may reach.  The
+// population pointers of a kernel that calls chain_wait(), and of what it
+// calls, are therefore plain; lists, rows, masks and tables keep the promise.
 __device__ __forceinline__ void chain_start() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

@@ -376,7 +376,7 @@ template <int D, int Q, class T, int V, bool SOLID, int XA, int XB>
 __device__ __forceinline__ void average_lanes(bool take, int ch, int P, int c, int g,
                                               const RowPos<D, V>& pos, const int32_t* nb,
                                               const uint64_t* sm, int flags,
-                                              const T* __restrict__ fch, T* __restrict__ fpar,
+                                              const T* fch, T* fpar,
                                               const int32_t* __restrict__ prow,
                                               const uint64_t* __restrict__ solidmask,
                                               typename Store<T>::R keep) {
@@ -479,7 +479,7 @@ __device__ __forceinline__ void gather_half(R (&out)[N / 2][2 * NIN], const R (&
 template <int D, int Q, class T, bool SOLID>
 __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     k_average(const int32_t* __restrict__ list, int64_t n_items, bool by_parent,
-              T* __restrict__ fpar, const T* __restrict__ fch, const int32_t* __restrict__ child0,
+              T* fpar, const T* fch, const int32_t* __restrict__ child0,
               const int32_t* __restrict__ parent, const uint64_t* __restrict__ cellmask,
               const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
               double ratio, int mode_sync) {
@@ -578,8 +578,8 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
 // 20 coarse steps).  Children are groups of N_c IDs from first_child on.
 template <int D, int Q, class T, bool SOLID>
 __global__ void __launch_bounds__(64, (average_min_ctas<Q, T, 64>()))
-    k_average_groups(const int32_t* __restrict__ items, int n, T* __restrict__ fpar,
-                     const T* __restrict__ fch, int first_child,
+    k_average_groups(const int32_t* __restrict__ items, int n, T* fpar,
+                     const T* fch, int first_child,
                      const int32_t* __restrict__ parent, const int32_t* __restrict__ nbr,
                      const uint64_t* __restrict__ solidmask, typename Store<T>::R keep) {
   constexpr int V = D == 3 ? 2 : 1;
