@@ -746,6 +746,18 @@ __device__ __forceinline__ void step_row(const T* gin, T* gout, int b,
   if constexpr (SOLID) {
     if (flags & BF_SOLID) solid = (unsigned)(sm[D == 2 ? 4 : 13] >> pos.l0) & ALL;
   }
+  if constexpr (SOLID && XCHG) {
+    // a solid cell is at rest; its slots, which no step writes, may hold what
+    // an earlier block of the same ID left there
+    if (par.rc && solid) {
+      static_for<0, Q>([&](auto P) {
+        constexpr double wp = VS<D, Q>::w[P];
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+          if ((solid >> i) & 1u) par.rc[P * M + pos.l0 + i] = SH ? R(0) : R(wp);
+      });
+    }
+  }
   if (!SOLID || solid == 0u) {
     static_for<0, Q>([&](auto P) { *reinterpret_cast<Vec<T, V>*>(own + P * M) = g[P]; });
   } else if (solid != ALL) {
