@@ -1281,6 +1281,26 @@ __global__ void k_init_rest(int64_t cap, T* __restrict__ f) {
   });
 }
 
+// The rest state in the own slots of the solid cells of the listed blocks.  No
+// step writes these slots, and an ID may have belonged to a fluid block before,
+// so they are set in both buffers when a block is made: here in the one that
+// the interpolation of new children does not fill.
+template <int D, int Q, class T>
+__global__ void k_solid_rest(const int32_t* __restrict__ list, int n,
+                             const uint64_t* __restrict__ solidmask, T* __restrict__ f) {
+  using R = typename Store<T>::R;
+  constexpr int M = Block<D>::M;
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= (int64_t)n * M) return;
+  const int b = __ldg(list + g / M), l = (int)(g % M);
+  if (!((__ldg(solidmask + b) >> l) & 1ull)) return;
+  const size_t own = (size_t)b * (Q * M) + l;
+  static_for<0, Q>([&](auto P) {
+    constexpr double wp = VS<D, Q>::w[P];
+    f[own + (size_t)P * M] = Store<T>::template save<D, Q, P>(R(wp));
+  });
+}
+
 // Adaptation: for every cell x of a child about to be removed and every link
 // p whose target y = x + c_p lies in a same-level block that stays, the value
 // stored in x's slot p is y's pre-collision f_p; once the block is gone y
@@ -1601,6 +1621,9 @@ struct Launch {
   static void init_rest(cudaStream_t s, int64_t cap, void* f) {
     k_init_rest<D, Q, T><<<grid_for(cap * M, 256), 256, 0, s>>>(cap, (T*)f);
   }
+  static void solid_rest(cudaStream_t s, const int32_t* list, int n, const uint64_t* sm, void* f) {
+    if (n > 0) k_solid_rest<D, Q, T><<<grid_for((int64_t)n * M, 256), 256, 0, s>>>(list, n, sm, (T*)f);
+  }
   static int mass_partial(cudaStream_t s, int64_t cap, const void* fa, const void* fb,
                           unsigned cur, const int32_t* level, const int32_t* status,
                           const int32_t* nbr, const uint64_t* sm, double* partial) {
@@ -1721,7 +1744,7 @@ struct Launch {
                              init_rest,     mass_partial,   force_partial,
                              collide_stream_batch, interp_batch, average_batch,
                              persistent_ctas, batch_persistent, features,
-                             coarsen_fixup};
+                             coarsen_fixup, solid_rest};
     return &o;
   }
 };

@@ -206,6 +206,8 @@ struct LbmOps {
                         const int32_t* parent, const int8_t* marks, const int32_t* nbr,
                         const uint64_t* solidmask, const int32_t* level, void* fa, void* fb,
                         unsigned cur);
+  // the rest state in the solid cells of the listed blocks, in buffer f
+  void (*solid_rest)(cudaStream_t, const int32_t* list, int n, const uint64_t* solidmask, void* f);
 };
 
 const LbmOps* lbm_ops_d2q9(int storage);

@@ -880,12 +880,15 @@ static int adapt_t(Instance* a, amr_adapt_stats* st) {
     const int64_t nnew = nRL[L] * NC;
     k_append_children<D><<<blocks_for(nnew), 256, 0, s>>>(C + offR[L], (int)nRL[L], a->child0, W);
     a->launches += 1;
-    if (a->solid)
+    if (a->solid) {
       k_solidmask<D><<<blocks_for(nnew), 256, 0, s>>>(W, (int)nnew, a->level, a->X,
                                                       a->cfg.solid[0], a->cfg.solid[1],
                                                       a->cfg.solid[2], a->cfg.solid[3],
                                                       a->solidmask);
+      a->ops->solid_rest(s, W, (int)nnew, a->solidmask, a->fbuf(L + 1, 1));
       a->launches += 1;
+    }
+    a->launches += 1;
     AMR_CUDA(cudaGetLastError());
     const double ratio = a->tau[L + 1] / (2.0 * a->tau[L]);
     a->ops->interp(s, C + offR[L], (int)nRL[L], a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->cellmask, a->nbr, a->sm(), a->parent, a->marks, ratio,

@@ -89,7 +89,7 @@ def test_the_sequence_reuses_partly_solid_parents(dim, q):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("dim,q", [(2, 9), (3, 19), (3, 27)])
-@pytest.mark.parametrize("interp", ["linear"])
+@pytest.mark.parametrize("interp", ["linear", "cubic"])
 def test_reused_blocks_at_a_solid(dim, q, interp):
     """FP64 within the bars of the other parity tests (1e-12 relative L2, 1e-10
     per cell), as a graph and launch by launch; FP16 and BF16 storage (the
