@@ -1528,17 +1528,14 @@ struct Launch {
     // kernel_variant: 1 / 2 / 3 / 4: CTAs of 512 / 256 / 128 / 64 cells (8 /
     // 4 / 2 / 1 blocks of 4^3 cells; never less than a warp); 5: 128 cells
     // with 128 more resident threads per SM (tighter register budget); 0
-    // (auto) and launches with exchanging parents: kAutoCells
-    if (x || prm.variant == 0 || prm.variant > 5) {
-      one_pass<SOLID, kAutoCells>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
-      return;
-    }
-    switch (prm.variant) {
+    // (auto), every other value, and launches with exchanging parents: kAutoCells
+    switch (x ? 0 : prm.variant) {
       case 1: one_pass<SOLID, 512>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 2: one_pass<SOLID, 256>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 3: one_pass<SOLID, 128>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 4: one_pass<SOLID, 64>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 5: one_pass<SOLID, 128, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
+      default: one_pass<SOLID, kAutoCells>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
     }
   }
 
