@@ -428,23 +428,27 @@ __device__ __forceinline__ Vec<T, V> ld_vec(const T* p) {
 // Four (two blocks per warp) were faster on the periodic 256^3 forest, where
 // every block takes the same path (0.37 against 0.40 ms per step), and slower
 // on the 64^3 cavity with three extra levels, where they differ (38.2 against
-// 36.1 ms for ten coarse steps).  2D: one; the meshes are small and latency
-// counts (128^2 cavity, FP32, 20 coarse steps: 1.9 / 2.2 / 3.0 ms with 1 / 2 / 4).
+// 36.1 ms for ten coarse steps).  FP64: one.  An FP64 instruction occupies a
+// scheduler for 64 cycles and an SM for 19, so an SM needs four warps to run at
+// its rate: two warps per block reach it with half the blocks (coarse steps of
+// cavities and prisms, one against two: 24^3 16.4 / 26.6 us, 24^3 with two extra
+// levels 658 / 773, 64^3 with one 579 / 612, 128x32x16 prism with three 3461 /
+// 3632; none slower).  2D: one; the meshes are small and latency counts (128^2
+// cavity, FP32, 20 coarse steps: 1.9 / 2.2 / 3.0 ms with 1 / 2 / 4).
 template <int D, class T>
 constexpr int row_cells() {
-  return D == 2 ? 1 : 2;
+  return D == 2 || sizeof(T) == 8 ? 1 : 2;
 }
 
-// Threads of a CTA that holds `cells` cells (at least a warp), and the CTAs
-// per SM its register budget is set for: 896 threads for D3Q19 in 32 bits and
+// Threads of a CTA that holds `cells` cells, V per thread (at least a warp), and
+// the CTAs per SM its register budget is set for: 896 threads for D3Q19 in 32 bits and
 // less (72 registers; the cavity above takes 37.0 / 36.1 / 36.3 ms with 768 /
 // 896 / 1024), 640 for D3Q27 (96 registers; 13.8 ms against 15.4 with 768 for
 // five coarse steps of the 128x32x32 prism in FP16), fewer for FP64, whose
 // arithmetic saturates with few warps.
-template <int D, class T>
+template <int V>
 constexpr int row_threads(int cells) {
-  const int n = cells / row_cells<D, T>();
-  return n < 32 ? 32 : n;
+  return cells / V < 32 ? 32 : cells / V;
 }
 template <int Q, class T, int THREADS, bool DENSE = false>
 constexpr int row_min_ctas() {
@@ -882,7 +886,9 @@ __device__ __forceinline__ void interp_rows(const typename Store<T>::R* rc, int 
 
 // One thread per V cells of an x-row (row_cells).  The threads of a block lie
 // in one warp, so staging its neighbour row, and handing a parent's rescaled
-// cells to its children's interpolation, need no CTA barrier.
+// cells to its children's interpolation, need no CTA barrier.  With one cell
+// per thread in 3D a block takes two warps: each stages the row for itself, and
+// the CTA, which then holds one block, meets before the interpolation.
 template <int D, int Q, class T, bool SOLID, int THREADS, int MIN_CTAS, bool GHOST_IN, bool XCHG>
 __global__ void __launch_bounds__(THREADS, MIN_CTAS)
     k_collide_stream(const int32_t* __restrict__ list, int n, const T* gin,
@@ -893,39 +899,42 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
   using R = typename Store<T>::R;
   constexpr int M = Block<D>::M;
   constexpr int V = row_cells<D, T>();
-  constexpr int TPB = M / V;
+  constexpr int TPB = M / V;                // threads of a block
+  constexpr int LPR = TPB < 32 ? TPB : 32;  // lanes that share a staged row
   constexpr int NCODE = D == 2 ? 9 : 27;
-  constexpr int BPC = THREADS / TPB;
-  static_assert(THREADS % 32 == 0 && 32 % TPB == 0, "the threads of a block lie in one warp");
-  __shared__ int32_t s_nb[BPC][NCODE];
-  __shared__ uint64_t s_sm[SOLID ? BPC : 1][SOLID ? NCODE : 1];
+  constexpr int BPC = THREADS / TPB, RPC = THREADS / LPR;
+  static_assert(THREADS % 32 == 0 && (32 % TPB == 0 || THREADS == TPB || !XCHG),
+                "the threads of an exchanging parent lie in one warp or fill the CTA");
+  __shared__ int32_t s_nb[RPC][NCODE];
+  __shared__ uint64_t s_sm[SOLID ? RPC : 1][SOLID ? NCODE : 1];
   __shared__ __align__(16) R s_rc[XCHG ? BPC : 1][XCHG ? Q * M : 1];   // rescaled parent cells
 
   chain_start();
-  const int slot = threadIdx.x / TPB;
+  const int slot = threadIdx.x / TPB, row = threadIdx.x / LPR;
   const int t = threadIdx.x % TPB;
   const int bi = blockIdx.x * BPC + slot;
   if (bi >= n) {                           // (the same for the threads of a block)
     chain_wait();
     return;
   }
-  const unsigned lanes = block_lanes<TPB>();
+  const unsigned lanes = block_lanes<LPR>();
   const int b = __ldg(list + bi);
   uint64_t ghost = 0ull;
   if constexpr (GHOST_IN) ghost = __ldg(cellmask + 2 * (size_t)b);
   int c0 = NONE;
   if constexpr (XCHG) c0 = __ldg(ex.child0 + b);
-  const int flags = stage_block<D, TPB, SOLID>(s_nb[slot], SOLID ? s_sm[slot] : nullptr, b, t,
+  const int flags = stage_block<D, LPR, SOLID>(s_nb[row], SOLID ? s_sm[row] : nullptr, b, t % LPR,
                                                lanes, nbr, solidmask, &prm.faces);
   chain_wait();
   ParentOut<R> par{nullptr, R(0)};
   if constexpr (XCHG) par = {c0 >= 0 ? s_rc[slot] : nullptr, ex.keep<R>()};
-  step_row<D, Q, T, V, SOLID, GHOST_IN, XCHG, false>(gin, gout, b, t, s_nb[slot],
-                                                     SOLID ? s_sm[slot] : nullptr, flags, ghost,
+  step_row<D, Q, T, V, SOLID, GHOST_IN, XCHG, false>(gin, gout, b, t, s_nb[row],
+                                                     SOLID ? s_sm[row] : nullptr, flags, ghost,
                                                      prm.rate<R>(), prm.faces, par);
   if constexpr (XCHG) {
     if (c0 >= 0) {
-      __syncwarp(lanes);
+      if constexpr (TPB > 32) __syncthreads();   // (one block: the same for the CTA)
+      else __syncwarp(lanes);
       interp_rows<D, Q, T, V>(s_rc[slot], t, c0, ex.cellmask, (T*)ex.fine_out, solidmask);
     }
   }

@@ -621,20 +621,20 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
                            const InstDesc* __restrict__ descs, int level, int which_in) {
   using R = typename Store<T>::R;
   constexpr int V = row_cells<D, T>();
-  constexpr int TPB = Block<D>::M / V;
+  constexpr int TPB = Block<D>::M / V, LPR = TPB < 32 ? TPB : 32;
   constexpr int BPC = THREADS / TPB;
-  __shared__ int32_t s_nb[BPC][D == 2 ? 9 : 27];
-  const int slot = threadIdx.x / TPB;
+  __shared__ int32_t s_nb[THREADS / LPR][D == 2 ? 9 : 27];
+  const int row = threadIdx.x / LPR;
   const int t = threadIdx.x % TPB;
-  const int bi = blockIdx.x * BPC + slot;
+  const int bi = blockIdx.x * BPC + threadIdx.x / TPB;
   if (bi >= n) return;
   const uint32_t it = __ldg(items + bi);
   const InstDesc& d = descs[it >> BATCH_SHIFT];
   const int b = (int)(it & BATCH_MASK);
-  const int flags = stage_block<D, TPB, false>(s_nb[slot], nullptr, b, t, block_lanes<TPB>(),
+  const int flags = stage_block<D, LPR, false>(s_nb[row], nullptr, b, t % LPR, block_lanes<LPR>(),
                                                d.nbr, nullptr, &d.faces);
   step_row<D, Q, T, V, false, false, false, false>(
-      (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[slot], nullptr, flags, 0ull,
+      (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[row], nullptr, flags, 0ull,
       R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
 }
 
@@ -731,23 +731,26 @@ __device__ __forceinline__ bool persist_wait(const uint32_t* cnt, uint32_t targe
 }
 
 // Collide-stream tile: `nblk` (<= PERSIST_MAX_TILE) active blocks of one
-// member, their rows spread over the CTA's threads.  The same step as
-// k_collide_stream_batch, with every population read from L2.
-template <int D, int Q, class T, int THREADS>
+// member, their rows spread over the CTA's threads, V cells each.  The same step
+// as k_collide_stream_batch, with every population read from L2.  `s_nb`: a row
+// for each warp, which takes a block (half of one with V = 1 in 3D) at a time.
+template <int D, int Q, class T, int THREADS, int V>
 __device__ __forceinline__ void persist_collide(const InstDesc& d, const uint32_t* items, int nblk,
                                                 int level, int which_in,
                                                 int32_t (*s_nb)[D == 2 ? 9 : 27]) {
   using R = typename Store<T>::R;
-  constexpr int V = row_cells<D, T>();
-  constexpr int TPB = Block<D>::M / V;
-  const int t = threadIdx.x % TPB;
-  for (int s = threadIdx.x / TPB; s < nblk; s += THREADS / TPB) {
-    const int b = (int)(__ldg(items + s) & BATCH_MASK);
-    const int flags = stage_block<D, TPB, false>(s_nb[s], nullptr, b, t, block_lanes<TPB>(),
+  constexpr int TPB = Block<D>::M / V, LPR = TPB < 32 ? TPB : 32;
+  constexpr int PARTS = TPB / LPR;      // of a block
+  int32_t* nb = s_nb[threadIdx.x / LPR];
+  for (int s = threadIdx.x / LPR; s < nblk * PARTS; s += THREADS / LPR) {
+    const int b = (int)(__ldg(items + s / PARTS) & BATCH_MASK);
+    const int t = s % PARTS * LPR + threadIdx.x % LPR;
+    const int flags = stage_block<D, LPR, false>(nb, nullptr, b, t % LPR, block_lanes<LPR>(),
                                                  d.nbr, nullptr, &d.faces);
     step_row<D, Q, T, V, false, false, false, true>(
-        (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, s_nb[s], nullptr, flags, 0ull,
+        (const T*)d.f[which_in], (T*)d.f[which_in ^ 1], b, t, nb, nullptr, flags, 0ull,
         R(d.omega[level]), d.faces, ParentOut<R>{nullptr, R(0)});
+    __syncwarp(block_lanes<LPR>());     // the row is done with
   }
 }
 
@@ -824,7 +827,7 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
   R (*sF)[Q][M] = reinterpret_cast<R (*)[Q][M]>(s_dyn);
   int32_t (*s_rows)[1 + NC][NK] =
       reinterpret_cast<int32_t (*)[1 + NC][NK]>(s_dyn + sizeof(R) * U * Q * M);
-  __shared__ int32_t s_nb[PERSIST_MAX_TILE][D == 2 ? 9 : 27];
+  __shared__ int32_t s_nb[THREADS / (D == 2 ? 16 : 32)][D == 2 ? 9 : 27];
   __shared__ long long s_take;
   __shared__ int32_t s_go;
   const long long total = (long long)a.tiles_per_step * a.n_steps;
@@ -890,7 +893,8 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
     if (op == PH_COLLIDE) {
       const int first = tile * a.tile_blocks;
       const int nblk = min(a.tile_blocks, ni - first);
-      persist_collide<D, Q, T, THREADS>(d, items + first, nblk, level, win, s_nb);
+      persist_collide<D, Q, T, THREADS, row_cells<D, T>()>(d, items + first, nblk, level, win,
+                                                           s_nb);
     } else if (op == PH_INTERP) {
       persist_interp<D, Q, T, THREADS>(d, items, ni, tile, level, win, wch, sF, s_rows);
     } else {
@@ -1488,7 +1492,8 @@ struct Launch {
   // cells per CTA.  2D meshes are small: CTAs of one or two warps spread them
   // over the SMs (an SM executes one FP64 warp instruction per 19 cycles; the
   // 64^2 FP64 cavity took 2.20 ms with 256 cells per CTA, 1.66 with 32)
-  static constexpr int kAutoCells = D == 3 ? 256 : (sizeof(T) == 8 ? 32 : 64);
+  static constexpr int kAutoCells = D == 3 ? (sizeof(T) == 8 ? 64 : 256)
+                                           : (sizeof(T) == 8 ? 32 : 64);
 
   static int setup() {
     int dev = 0, sms = 0;
@@ -1498,12 +1503,13 @@ struct Launch {
     return 0;
   }
 
-  // CELLS cells per CTA (at least the blocks of a warp)
-  template <bool SOLID, int CELLS, bool DENSE = false>
+  // CELLS cells per CTA (at least the blocks of a warp); XCHG:
+  // instantiated for launches with exchanging parents as well
+  template <bool SOLID, int CELLS, bool XCHG, bool DENSE = false>
   static void one_pass(cudaStream_t s, const int32_t* list, int n, const void* fin, void* fout,
                        const int32_t* nbr, const uint64_t* sm, const StepParams& prm,
                        const uint64_t* gm, const Exchange* xchg) {
-    constexpr int THREADS = row_threads<D, T>(CELLS);
+    constexpr int V = row_cells<D, T>(), THREADS = row_threads<V>(CELLS);
     constexpr int MIN = row_min_ctas<Q, T, THREADS, DENSE>();
     const T* in = (const T*)fin;
     T* out = (T*)fout;
@@ -1511,13 +1517,15 @@ struct Launch {
     if (xchg) ex = *xchg;
     auto launch = [&](auto ghost, auto parents) {
       constexpr bool G = decltype(ghost)::value, X = decltype(parents)::value;
-      const int grid = grid_for(n, THREADS * row_cells<D, T>() / M);
+      const int grid = grid_for(n, THREADS * V / M);
       launch_chained(k_collide_stream<D, Q, T, SOLID, THREADS, MIN, G, X>, prm.chained, grid,
                      THREADS, s, list, n, in, out, nbr, sm, prm, gm, ex);
     };
-    if (gm && xchg) launch(std::true_type{}, std::true_type{});
-    else if (gm) launch(std::true_type{}, std::false_type{});
-    else if (xchg) launch(std::false_type{}, std::true_type{});
+    if constexpr (XCHG) {
+      if (gm && xchg) return launch(std::true_type{}, std::true_type{});
+      if (xchg) return launch(std::false_type{}, std::true_type{});
+    }
+    if (gm) launch(std::true_type{}, std::false_type{});
     else launch(std::false_type{}, std::false_type{});
   }
 
@@ -1530,12 +1538,15 @@ struct Launch {
     // with 128 more resident threads per SM (tighter register budget); 0
     // (auto), every other value, and launches with exchanging parents: kAutoCells
     switch (x ? 0 : prm.variant) {
-      case 1: one_pass<SOLID, 512>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      case 2: one_pass<SOLID, 256>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      case 3: one_pass<SOLID, 128>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      case 4: one_pass<SOLID, 64>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      case 5: one_pass<SOLID, 128, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
-      default: one_pass<SOLID, kAutoCells>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
+      case 1: one_pass<SOLID, 512, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
+      case 2: one_pass<SOLID, 256, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
+      case 3: one_pass<SOLID, 128, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
+      case 4: one_pass<SOLID, 64, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
+      case 5:
+        one_pass<SOLID, 128, false, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr);
+        break;
+      default:
+        one_pass<SOLID, kAutoCells, true>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
     }
   }
 
@@ -1670,10 +1681,9 @@ struct Launch {
   template <int CELLS>
   static void batch_cells(cudaStream_t s, const uint32_t* items, int n, const InstDesc* descs,
                           int level, int which_in) {
-    constexpr int THREADS = row_threads<D, T>(CELLS);
+    constexpr int V = row_cells<D, T>(), THREADS = row_threads<V>(CELLS);
     k_collide_stream_batch<D, Q, T, THREADS>
-        <<<grid_for(n, THREADS * row_cells<D, T>() / M), THREADS, 0, s>>>(items, n, descs, level,
-                                                                          which_in);
+        <<<grid_for(n, THREADS * V / M), THREADS, 0, s>>>(items, n, descs, level, which_in);
   }
   static void interp_batch(cudaStream_t s, const uint32_t* items, int n, const InstDesc* descs,
                            int level, int which_par, int which_ch) {
