@@ -352,14 +352,14 @@ static void advance(Instance* a, int L, bool first) {
       const double cells = (double)a->n_iface_cells[L];
       ProfScope ps(a, PK_AVERAGE, cells * (1.0 + 1.0 / a->nc) * a->q * a->elem, cells);
       // cubic interpolation samples every cell of the parent, so with it the
-      // parent cells over interior children are averaged as well (mode 1:
-      // every cell whose children are not ghosts), else only those over
-      // interface children: the groups of interface cells of the fine
-      // level's boundary blocks, listed at adaptation
+      // parent cells over interior children are averaged as well (every cell
+      // whose children are not ghosts), else only those over interface
+      // children: the groups of interface cells of the fine level's boundary
+      // blocks, listed at adaptation
       if (cubic)
         a->ops->average(a->stream, a->parents + (size_t)L * a->cap, (int)np, true,
                         a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                        a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid,
+                        a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), a->solid,
                         a->chained(np * a->M * a->nc));
       else
         a->ops->average_groups(a->stream, a->agrp + a->agrp_off[L + 1], (int)a->n_agrp[L + 1],
@@ -460,7 +460,7 @@ static void level_sync(Instance* a) {
     // every block of level L + 1 is the child of a refined block
     a->ops->average(a->stream, a->order + (size_t)(L + 1) * a->cap, (int)a->n_ids[L + 1], false,
                     a->fbuf(L, 0), a->fbuf(L + 1, 0), a->child0, a->parent,
-                    a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), 1, a->solid, false);
+                    a->cellmask, a->nbr, a->sm(), ratio_fc(a, L), a->solid, false);
     a->launches += 1;
   }
   for (int L = 0; L + 1 < a->lmax; ++L) {

@@ -37,7 +37,7 @@ struct Batch {
           n_ids[BATCH_MAX_LEVELS] = {};
   int64_t list_cap = 0;
   unsigned cur = 0;
-  int variant = 512;   // threads per CTA of the batched collide-stream
+  int variant = 512;   // cells per CTA of the batched collide-stream
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   bool graph_valid = false;
   int64_t launches = 0, graph_launches[2] = {0, 0};
@@ -678,7 +678,7 @@ int amr_batch_autotune(amr_batch_t* h, int trial_steps, int forms, amr_batch_con
   Batch* b = reinterpret_cast<Batch*>(h);
   if (!b || trial_steps < 1 || forms < 1 || forms > 7) return AMR_E_INVAL;
   // candidates in the order of ms_out: the graph form with 512 / 256 / 128 /
-  // 64 threads per CTA (M_L = 8 / 4 / 2 / 1 blocks per CTA in 3D), then the
+  // 64 cells per CTA (M_L = 8 / 4 / 2 / 1 blocks per CTA in 3D), then the
   // persistent form with M_L = 1, 2, 4, 8 blocks per tile x 64, 128, 256
   // threads per CTA, then the member-graph form
   std::vector<amr_batch_config_t> cand;

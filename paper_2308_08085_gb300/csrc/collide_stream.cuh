@@ -493,13 +493,11 @@ struct RowPos {
   // the value beside the vector for c_x = CX: x of its cell, code step
   template <int CX>
   __device__ __forceinline__ int edge_x() const {
-    if constexpr (V == 4) return CX > 0 ? 3 : 0;
-    else return CX > 0 ? (i0 - 1) & 3 : (i0 + V) & 3;
+    return CX > 0 ? (i0 - 1) & 3 : (i0 + V) & 3;
   }
   template <int CX>
   __device__ __forceinline__ int edge_code() const {
-    if constexpr (V == 4) return CX > 0 ? -1 : 1;
-    else return CX > 0 ? (i0 == 0 ? -1 : 0) : (i0 + V == 4 ? 1 : 0);
+    return CX > 0 ? (i0 == 0 ? -1 : 0) : (i0 + V == 4 ? 1 : 0);
   }
 };
 

@@ -287,27 +287,28 @@ __global__ void __launch_bounds__(64, sizeof(typename Store<T>::R) == 8 ? 5 : 10
 // ===================================================== fine-to-coarse averaging
 // Section 3.4.3.  A child covers 2^D parent cells (g = gx + 2 gy [+ 4 gz]),
 // each the mean of a 2^D group of the child's fine cells, which share one
-// class.  A group is taken when its cells are interface cells (mode_sync = 0)
-// or not ghosts (mode_sync = 1), and its parent cell is not solid.  One thread
-// per fine cell gathers it and rescales it to the coarse level
-// (f_eq + (f - f_eq) r) into shared memory; then one thread per taken group
-// sums its 2^D cells and scatters the mean into the parent cell.
+// class.  The level step takes the groups of interface cells, the
+// synchronisation (and the level step with cubic interpolation) every group
+// that is not of ghosts; the parent cell must not be solid.
+
+// The first cell of group g of a child.
 template <int D>
-__device__ __forceinline__ bool average_group_taken(const uint64_t* __restrict__ cellmask, int ch,
-                                                    int g, int mode_sync) {
-  const int f0 = Block<D>::cell(2 * (g & 1), 2 * ((g >> 1) & 1), 2 * ((g >> 2) & 1));
-  if (mode_sync) return !((__ldg(cellmask + 2 * (size_t)ch) >> f0) & 1ull);
-  return (__ldg(cellmask + 2 * (size_t)ch + 1) >> f0) & 1ull;
+__device__ __forceinline__ int group_cell(int g) {
+  return Block<D>::cell(2 * (g & 1), 2 * ((g >> 1) & 1), 2 * ((g >> 2) & 1));
 }
 
-template <int D, int Q, class T, bool SOLID, bool COH = false>
+// The batched forms' averaging, by interface groups: one thread per fine cell
+// gathers it and rescales it to the coarse level (f_eq + (f - f_eq) r) into
+// shared memory; then one thread per taken group sums its 2^D cells and
+// scatters the mean into the parent cell.
+
+template <int D, int Q, class T, bool COH = false>
 __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D>::M],
                                               bool valid, int P, int c, int ch,
                                               int l, T* __restrict__ fpar,
                                               const T* __restrict__ fch, const uint64_t* __restrict__ cellmask,
                                               const int32_t* crow, const int32_t* prow,
-                                              const uint64_t* __restrict__ solidmask,
-                                              double ratio, int mode_sync) {
+                                              double ratio) {
   using S = Store<T>;
   using R = typename S::R;
   constexpr int M = Block<D>::M;
@@ -318,14 +319,12 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
     return Block<D>::cell(2 * (c & 1) + (gg & 1), 2 * ((c >> 1) & 1) + ((gg >> 1) & 1),
                           2 * ((c >> 2) & 1) + ((gg >> 2) & 1));
   };
-  // group gg is taken: its class matches and its parent cell is not solid
   auto taken = [&](int gg) {
-    return average_group_taken<D>(cellmask, ch, gg, mode_sync) &&
-           !(SOLID && solidmask && ((__ldg(solidmask + P) >> parent_cell(gg)) & 1ull));
+    return (__ldg(cellmask + 2 * (size_t)ch + 1) >> group_cell<D>(gg)) & 1ull;
   };
   if (valid && taken(g)) {
     R f[Q];
-    gather_cell<D, Q, T, SOLID, COH>(f, fch, ch, l, crow, solidmask);
+    gather_cell<D, Q, T, false, COH>(f, fch, ch, l, crow, nullptr);
     R rho, ux, uy, uz;
     moments<D, Q>(f, rho, ux, uy, uz);
     const R usq15 = R(1.5) * (ux * ux + uy * uy + uz * uz);
@@ -339,7 +338,7 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
   // one thread per taken group: the mean of its 2^D rescaled cells,
   // scattered into the parent cell
   if (valid && l < NC && taken(l)) {
-    const int f0 = Block<D>::cell(2 * (l & 1), 2 * ((l >> 1) & 1), 2 * ((l >> 2) & 1));
+    const int f0 = group_cell<D>(l);
     R acc[Q];
     const R inv = R(1) / R(NC);
     static_for<0, Q>([&](auto Pp) {
@@ -348,7 +347,7 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
       for (int s = 0; s < NC; ++s) a += sR[Pp][f0 + Block<D>::cell(s & 1, (s >> 1) & 1, (s >> 2) & 1)];
       acc[Pp] = a * inv;
     });
-    scatter_cell<D, Q, T, SOLID>(acc, fpar, P, parent_cell(l), prow, solidmask);
+    scatter_cell<D, Q, T, false>(acc, fpar, P, parent_cell(l), prow, nullptr);
   }
 }
 
@@ -363,7 +362,7 @@ constexpr int average_min_ctas() {
   return (Q == 9 ? 1024 : (sizeof(T) == 8 ? 384 : (Q == 27 ? 768 : 1024))) / THREADS;
 }
 
-// The averaging of a child's cells by x-pairs (3D; by cells in 2D): each of
+// The averaging of a group's cells by x-pairs (3D; by cells in 2D): each of
 // the four lanes of a group holds V of its 2^D cells, gathers and rescales
 // them (f_eq + (f - f_eq) r = f + (f_eq - f)(1 - r), Section 3.4.3), sums them, and
 // the lanes XA and XB apart sum theirs with a reduce-scatter: at each
@@ -475,14 +474,14 @@ __device__ __forceinline__ void gather_half(R (&out)[N / 2][2 * NIN], const R (&
 // and inference of a 90,000-block cavity, D3Q19 FP32: 0.93 ms; 0.88 with sums
 // by pairs here and in k_features, 1.40 with a thread per cell.
 // by_parent: child item i is child i % N_c of list[i / N_c]; else it is the
-// block list[i].  mode_sync as in average_group_taken.
+// block list[i].  Every group of non-ghost cells is taken.
 template <int D, int Q, class T, bool SOLID>
 __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     k_average(const int32_t* __restrict__ list, int64_t n_items, bool by_parent,
               T* fpar, const T* fch, const int32_t* __restrict__ child0,
               const int32_t* __restrict__ parent, const uint64_t* __restrict__ cellmask,
               const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
-              double ratio, int mode_sync) {
+              double ratio) {
   using S = Store<T>;
   using R = typename S::R;
   constexpr int V = D == 3 ? 2 : 1;
@@ -511,7 +510,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
       P = __ldg(parent + ch);
       c = ch - __ldg(child0 + P);
     }
-    take = average_group_taken<D>(cellmask, ch, g, mode_sync);
+    take = !((__ldg(cellmask + 2 * (size_t)ch) >> group_cell<D>(g)) & 1ull);
     if (SOLID && take) {
       const int pc = Block<D>::cell(2 * (c & 1) + (g & 1), 2 * ((c >> 1) & 1) + ((g >> 1) & 1),
                                     2 * ((c >> 2) & 1) + ((g >> 2) & 1));
@@ -702,9 +701,9 @@ __global__ void __launch_bounds__(128)
   stage_row<D>(s_row[slot][0], d.nbr, valid ? ch : NONE, l, M);
   stage_row<D>(s_row[slot][1], d.nbr, valid ? P : NONE, l, M);
   __syncthreads();
-  average_child<D, Q, T, false>(sR[slot], valid, P, c, ch, l, (T*)d.f[which_par],
-                                (const T*)d.f[which_ch], d.cellmask, s_row[slot][0],
-                                s_row[slot][1], nullptr, d.r_fc[level], 0);
+  average_child<D, Q, T>(sR[slot], valid, P, c, ch, l, (T*)d.f[which_par],
+                         (const T*)d.f[which_ch], d.cellmask, s_row[slot][0], s_row[slot][1],
+                         d.r_fc[level]);
 }
 
 // ============================ batched instances: persistent form (PersistArgs)
@@ -807,9 +806,9 @@ __device__ __noinline__ void persist_average(const InstDesc& d, const uint32_t* 
   stage_row<D>(s_rows[slot][0], d.nbr, valid ? ch : NONE, l, M);
   stage_row<D>(s_rows[slot][1], d.nbr, valid ? P : NONE, l, M);
   __syncthreads();
-  average_child<D, Q, T, false, true>(sF[slot], valid, P, c, ch, l, (T*)d.f[win],
-                                      (const T*)d.f[wch], d.cellmask, s_rows[slot][0],
-                                      s_rows[slot][1], nullptr, d.r_fc[level], 0);
+  average_child<D, Q, T, true>(sF[slot], valid, P, c, ch, l, (T*)d.f[win],
+                               (const T*)d.f[wch], d.cellmask, s_rows[slot][0], s_rows[slot][1],
+                               d.r_fc[level]);
 }
 
 // The persistent kernel.  Dynamic shared memory: the rescaled populations of
@@ -1418,24 +1417,19 @@ __global__ void __launch_bounds__(256)
   using R = typename S::R;
   constexpr int M = Block<D>::M;
   constexpr int NCODE = D == 2 ? 9 : 27, CENTER = D == 2 ? 4 : 13;
-  __shared__ int32_t s_nb[8][NCODE];
   __shared__ uint64_t s_sm[8][NCODE];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double acc[3] = {0.0, 0.0, 0.0};
   for (int bi = blockIdx.x * 8 + warp; bi < n; bi += gridDim.x * 8) {
     const int b = __ldg(list + bi);
-    int v = NONE;
     uint64_t m = 0ull;
     if (lane < NCODE) {
-      v = __ldg(nbr + (size_t)b * NBR_STRIDE + geo_to_k<D>(lane));
+      const int v = __ldg(nbr + (size_t)b * NBR_STRIDE + geo_to_k<D>(lane));
       if (v >= 0) m = __ldg(solidmask + v);
     }
     if (!__any_sync(0xffffffffu, m != 0ull) || __ldg(status + b) != ST_UNREFINED) continue;
     __syncwarp();
-    if (lane < NCODE) {
-      s_nb[warp][lane] = v;
-      s_sm[warp][lane] = m;
-    }
+    if (lane < NCODE) s_sm[warp][lane] = m;
     __syncwarp();
     for (int l = lane; l < M; l += 32) {
       if ((s_sm[warp][CENTER] >> l) & 1ull) continue;
@@ -1592,15 +1586,15 @@ struct Launch {
   static void average(cudaStream_t s, const int32_t* list, int n, bool by_parent, void* fpar,
                       const void* fch, const int32_t* child0,
                       const int32_t* parent, const uint64_t* nm,
-                      const int32_t* nbr, const uint64_t* sm, double ratio, int mode_sync,
-                      bool solid, bool chained) {
+                      const int32_t* nbr, const uint64_t* sm, double ratio, bool solid,
+                      bool chained) {
     if (n <= 0) return;
     constexpr int CPC = 128 / (M / (D == 3 ? 2 : 1));
     const int64_t items = by_parent ? (int64_t)n * Block<D>::NC : (int64_t)n;
     const int grid = (int)((items + CPC - 1) / CPC);
     launch_chained(solid ? k_average<D, Q, T, true> : k_average<D, Q, T, false>, chained, grid,
                    128, s, list, items, by_parent, (T*)fpar, (const T*)fch, child0, parent, nm,
-                   nbr, solid ? sm : nullptr, ratio, mode_sync);
+                   nbr, solid ? sm : nullptr, ratio);
   }
   static void criterion(cudaStream_t s, const int32_t* list, int n, const void* f, const int32_t* nbr, const uint64_t* sm, const int32_t* status, int level,
                         int lmax, double inv_dx, int ns, int ni, int8_t* marks, double* w2out) {

@@ -141,18 +141,16 @@ struct LbmOps {
                  const int32_t* child0, const uint64_t* cellmask,
                  const int32_t* nbr, const uint64_t* solidmask, const int32_t* parent,
                  const int8_t* marks, double ratio, int mode, bool solid);
-  // fine-to-coarse averaging: by_parent -- `list` holds refined blocks, all
-  // their children are visited; else `list` holds children and parent[] leads
-  // to their parents.  mode 0: parent cells over interface children, 1: over
-  // every non-ghost child
+  // fine-to-coarse averaging of every non-ghost child cell: by_parent --
+  // `list` holds refined blocks, all their children are visited; else `list`
+  // holds children and parent[] leads to their parents
   void (*average)(cudaStream_t, const int32_t* list, int n, bool by_parent, void* fpar,
                   const void* fch, const int32_t* child0, const int32_t* parent,
                   const uint64_t* cellmask, const int32_t* nbr,
-                  const uint64_t* solidmask, double ratio, int mode_sync, bool solid,
-                  bool chained);
+                  const uint64_t* solidmask, double ratio, bool solid, bool chained);
   // the averaging of the level step over (block << 3 | group) items: the
   // groups of 2^D interface cells of the fine level's boundary blocks, each
-  // into its parent cell (the work of average mode 0, listed in advance);
+  // into its parent cell (listed in advance);
   // children are groups of 2^D IDs from first_child on
   void (*average_groups)(cudaStream_t, const int32_t* items, int n, void* fpar, const void* fch,
                          int64_t first_child, const int32_t* parent,
