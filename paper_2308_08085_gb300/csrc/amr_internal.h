@@ -94,8 +94,21 @@ struct Instance {
   // chaining, 34.9 with this limit, 35.6 with none; prism D3Q27 FP32 cubic:
   // 17.9 / 17.8 / 26.7 (most of that from its interpolation launches, which
   // are not chained at all now); 128^2 FP32 cavity, all launches small: 1.91 -> 1.61).
+  // FP64 launches are bound by the arithmetic of the busiest SM, and a dependent
+  // launch is placed around what its predecessor still holds, unevenly: none of
+  // a 3D FP64 coarse step is chained (29 forests of 24^3 to 128x32x16 root
+  // cells: 0 to 16 % slower), and all of a 2D one or nothing, by its cell
+  // updates (273 forests: up to 2^18 updates 7 % faster in the mean and at most
+  // 1 % slower, from there to 390,000 8 % either way, above up to 30 % slower).
   static constexpr int64_t kChainCells = int64_t(1) << 17;
+  static constexpr int64_t kChainUpdates64 = int64_t(1) << 18;
   int chain = 0;
+  bool may_chain() const {
+    if (elem != 8) return true;
+    int64_t updates = 0;
+    for (int L = 0; L < lmax; ++L) updates += (n_active[L] * M) << L;
+    return dim == 2 && updates <= kChainUpdates64;
+  }
   bool chained(int64_t cells) {
     const bool c = chain == 2 && cells <= kChainCells;
     if (chain) chain = 2;

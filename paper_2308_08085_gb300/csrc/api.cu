@@ -382,7 +382,7 @@ int64_t coarse_step_into(Instance* a, cudaStream_t s, int parity) {
   a->stream = s;
   a->profiling = 0;
   a->cur = (saved & ~1u) | (unsigned)parity;
-  a->chain = 1;
+  a->chain = a->may_chain() ? 1 : 0;
   const int64_t before = a->launches;
   advance(a, 0, false);
   a->chain = 0;
@@ -426,7 +426,8 @@ static int build_graphs(Handle* h) {
     if (e == cudaSuccess) {
       h->capturing = true;
       h->capture_parity = parity;
-      h->chain = h->profiling == 0 ? 1 : 0;   // (event nodes between the launches otherwise)
+      // (no chain where event nodes lie between the launches)
+      h->chain = h->profiling == 0 && h->may_chain() ? 1 : 0;
       const int64_t before = h->launches;
       advance(h, 0, false);
       h->chain = 0;
