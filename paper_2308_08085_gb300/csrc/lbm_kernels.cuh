@@ -1488,6 +1488,10 @@ struct Launch {
   // 64^2 FP64 cavity took 2.20 ms with 256 cells per CTA, 1.66 with 32)
   static constexpr int kAutoCells = D == 3 ? (sizeof(T) == 8 ? 64 : 256)
                                            : (sizeof(T) == 8 ? 32 : 64);
+  // ... 2D FP32 launches above this many cells: CTAs of 128 (one level, us per
+  // step with 64 / 128 cells: 512^2 8.3 / 8.3, 768^2 12.4 / 10.4, 1024^2 20.6 /
+  // 16.6, 2048^2 71.8 / 63.6, 3072^2 153.8 / 134.9)
+  static constexpr int64_t kWideCells = int64_t(1) << 18;
 
   static int setup() {
     int dev = 0, sms = 0;
@@ -1540,6 +1544,12 @@ struct Launch {
         one_pass<SOLID, 128, false, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr);
         break;
       default:
+        if constexpr (D == 2 && sizeof(T) == 4) {
+          if ((int64_t)n * M > kWideCells) {
+            one_pass<SOLID, 128, true>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
+            break;
+          }
+        }
         one_pass<SOLID, kAutoCells, true>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
     }
   }
