@@ -811,11 +811,27 @@ __device__ __noinline__ void persist_average(const InstDesc& d, const uint32_t* 
                                d.r_fc[level]);
 }
 
+// CTAs per SM of the persistent kernel: the interpolation and averaging tiles
+// and tiles smaller than the CTA leave threads idle, so larger CTAs are given
+// more of them than the collide-stream's budget (threads per SM for CTAs of 64 /
+// 128 / 256; three batches of 4 to 14 cavities, D3Q19 FP32, the largest tile of
+// each, ms per two steps with 896 / 1024 / 1280 / 1536: CTAs of 64 1.19 / 1.21 /
+// 1.39 / 2.04, of 128 1.24 / 1.16 / 1.19 / 1.38, of 256 1.47 / 1.31 / 1.28 / 1.39).
+template <int Q, class T, int THREADS>
+constexpr int persist_min_ctas() {
+  constexpr int size = THREADS == 64 ? 0 : (THREADS == 128 ? 1 : 2);
+  constexpr int f64[3][3] = {{1024, 1024, 1024}, {512, 512, 768}, {384, 384, 512}};
+  constexpr int f32[3][3] = {{1152, 1280, 1536}, {896, 1024, 1280},
+                             {704, sizeof(T) == 2 ? 768 : 896, sizeof(T) == 2 ? 768 : 1024}};
+  constexpr int q = Q == 9 ? 0 : (Q == 19 ? 1 : 2);
+  return (sizeof(T) == 8 ? f64 : f32)[q][size] / THREADS;
+}
+
 // The persistent kernel.  Dynamic shared memory: the rescaled populations of
 // the THREADS / M parents (interpolation) or children (averaging) of a tile,
 // then their neighbour rows.
 template <int D, int Q, class T, int THREADS>
-__global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
+__global__ void __launch_bounds__(THREADS, (persist_min_ctas<Q, T, THREADS>()))
     k_batch_persistent(PersistArgs a) {
   using R = typename Store<T>::R;
   constexpr int M = Block<D>::M;
@@ -892,8 +908,14 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
     if (op == PH_COLLIDE) {
       const int first = tile * a.tile_blocks;
       const int nblk = min(a.tile_blocks, ni - first);
-      persist_collide<D, Q, T, THREADS, row_cells<D, T>()>(d, items + first, nblk, level, win,
-                                                           s_nb);
+      // a cell per thread where two would leave half of the warps without work
+      // (the batch above, CTAs of 256 with tiles of one block: 5.1 ms against
+      // 3.3 with this and the budget)
+      if (row_cells<D, T>() == 1 || 2 * nblk * 32 <= THREADS)
+        persist_collide<D, Q, T, THREADS, 1>(d, items + first, nblk, level, win, s_nb);
+      else
+        persist_collide<D, Q, T, THREADS, row_cells<D, T>()>(d, items + first, nblk, level, win,
+                                                             s_nb);
     } else if (op == PH_INTERP) {
       persist_interp<D, Q, T, THREADS>(d, items, ni, tile, level, win, wch, sF, s_rows);
     } else {
