@@ -246,10 +246,13 @@ __global__ void __launch_bounds__(64)
   __shared__ __align__(16) float sW2[H][H];
   __shared__ float sb1[H], sb2[H], sw3[H];
   const int t = threadIdx.x;
+  // (many weights in flight: a CTA of 64 threads waits for each round of loads)
+#pragma unroll 14
   for (int i = t; i < H * 28; i += 64) {
     const int r = i / 28, c = i - r * 28;
     sW1[r][c] = c < IN ? __half2float(Ph[OW1 + r * IN + c]) : 0.f;
   }
+#pragma unroll 16
   for (int i = t; i < H * H; i += 64) sW2[i >> 6][i & 63] = __half2float(Ph[OW2 + i]);
   sb1[t] = __half2float(Ph[OB1 + t]);
   sb2[t] = __half2float(Ph[OB2 + t]);
