@@ -52,14 +52,17 @@ __device__ inline float softplus(float t) { return t > 0.f ? t + log1pf(expf(-t)
 // Summed gradient and loss over the samples of one minibatch.  A CTA of 256
 // threads takes tiles of S samples: the four groups of 64 threads compute
 // hidden unit t % 64 of S / 4 samples each, then every thread owns 16 entries
-// of dW2 and up to 7 of dW1 in registers, summed over its CTA's tiles and
-// added to `grad` once.  A minibatch of 1024 is latency-bound: 32 CTAs of 64
-// threads with 32 samples in a row took 88 us, 128 to 256 CTAs with one tile
-// each spread the serial chain of a sample over the chip.  Rows of W2 have a stride of
-// 65 words in shared memory (W1: 27), so that both W x and W^T x read without
-// bank conflicts.  The losses of a cluster of eight CTAs are summed before they
-// are added to *loss, whose FP32 sum over an epoch loses digits with every
-// addition.  Sample position pos maps to index (pos * mul + off) mod n,
+// of dW2 and up to 7 of dW1 in registers, summed over its CTA's tiles.  A
+// minibatch of 1024 is latency-bound: 32 CTAs of 64 threads with 32 samples in a
+// row took 88 us, 128 to 256 CTAs with one tile each spread the serial chain of
+// a sample over the chip (21 us).  Rows of W2 have a stride of 65 words in shared
+// memory (W1: 27), so that both W x and W^T x read without bank conflicts.
+// Gradient and loss lose digits with every addition to `grad` and *loss (256
+// additions of 4 samples each: relative error of the gradient 2.3e-7, 32 of 32:
+// 1.0e-7), so a cluster of eight CTAs is summed first, each CTA an eighth of the
+// entries out of the others' shared memory: 1.0e-7, 9e-8 at 8,192 samples, and
+// an eighth of the atomic additions (an epoch of 32 minibatches and its check
+// 755 -> 691 us).  Sample position pos maps to index (pos * mul + off) mod n,
 // a bijection when gcd(mul, n) = 1.
 constexpr int GT = 256, GC = 8;   // threads of a CTA, CTAs of a cluster
 template <int S>
@@ -68,8 +71,9 @@ __global__ void __cluster_dims__(GC, 1, 1) __launch_bounds__(GT)
            int64_t n, int64_t b0, int64_t bn, int64_t mul, int64_t off,
            float pos_weight, float* __restrict__ grad, float* __restrict__ loss) {
   constexpr int SPG = S / 4;                       // samples of a group
-  __shared__ float sW1[H * IN];
-  __shared__ float sW2[H * (H + 1)];
+  constexpr int NW = H * IN + H * (H + 1);
+  __shared__ float sP[NW > NP ? NW : NP];          // weights, then the CTA's gradient
+  float *sW1 = sP, *sW2 = sP + H * IN;
   __shared__ float sx[S][IN + 1], sy[S], sdz[S];
   __shared__ __align__(16) float sh1[S][H], sh2[S][H], sd1[S][H], sd2[S][H];
   __shared__ float sred[S][2];
@@ -183,31 +187,36 @@ __global__ void __cluster_dims__(GC, 1, 1) __launch_bounds__(GT)
   }
   __shared__ float s_loss;
   if (t == 0) s_loss = lsum;
-  auto cluster = cooperative_groups::this_cluster();
-  cluster.sync();
-  if (cluster.block_rank() == 0 && t == 0) {
-    float v = 0.f;
-    for (int r = 0; r < GC; ++r) v += *cluster.map_shared_rank(&s_loss, r);
-    atomicAdd(loss, v);
-  }
-  if (busy) {
-    // through shared memory, so that neighbouring lanes add to neighbouring words
+  if (busy) {                                      // (the weights are done with)
 #pragma unroll
-    for (int j = 0; j < 16; ++j) sW2[row * H + c2 + j] = gW2[j];
+    for (int j = 0; j < 16; ++j) sP[OW2 + row * H + c2 + j] = gW2[j];
 #pragma unroll
     for (int i = 0; i < 7; ++i)
-      if (c1 + i < IN) sW1[row * IN + c1 + i] = gW1[i];
-    __syncthreads();
-    for (int i = t; i < H * H; i += GT) atomicAdd(grad + OW2 + i, sW2[i]);
-    for (int i = t; i < H * IN; i += GT) atomicAdd(grad + OW1 + i, sW1[i]);
+      if (c1 + i < IN) sP[OW1 + row * IN + c1 + i] = gW1[i];
     if (t < H) {
-      atomicAdd(grad + OB1 + t, gb1);
-      atomicAdd(grad + OB2 + t, gb2);
-      atomicAdd(grad + OW3 + t, gw3);
+      sP[OB1 + t] = gb1;
+      sP[OB2 + t] = gb2;
+      sP[OW3 + t] = gw3;
     }
-    if (t == 0) atomicAdd(grad + OB3, gb3);
+    if (t == 0) sP[OB3] = gb3;
   }
-  cluster.sync();                                  // s_loss outlives its readers
+  auto cluster = cooperative_groups::this_cluster();
+  cluster.sync();
+  const int rank = (int)cluster.block_rank();
+  // CTAs of this cluster that had a tile (the first always)
+  const int64_t rest = (bn + S - 1) / S - (int64_t)(blockIdx.x - rank);
+  const int live = rest < GC ? (int)rest : GC;
+  for (int i = rank * GT + t; i < NP; i += GC * GT) {
+    float v = 0.f;
+    for (int r = 0; r < live; ++r) v += *cluster.map_shared_rank(&sP[i], r);
+    atomicAdd(grad + i, v);
+  }
+  if (rank == 0 && t == 0) {
+    float v = 0.f;
+    for (int r = 0; r < live; ++r) v += *cluster.map_shared_rank(&s_loss, r);
+    atomicAdd(loss, v);
+  }
+  cluster.sync();                                  // shared memory outlives its readers
 }
 
 // `clear`: leave the gradient zeroed for the next minibatch.
