@@ -352,11 +352,10 @@ __device__ __forceinline__ void average_child(typename Store<T>::R (*sR)[Block<D
 }
 
 // CTAs of THREADS threads per SM the register budget of the averaging (and of
-// the criterion, the summaries and the export of moments, which hold as much)
-// is set for: 1024 threads for D3Q19 (64 registers), 768 for D3Q27 (80).
-// Measured (marks and summaries of a cavity, D3Q19 / prism with cubic
-// interpolation, D3Q27): 0.91 / 17.8 ms with 768 / 512 threads, 0.88 / 16.9
-// with these, 0.94 / 17.1 with 1152 / 896 (spills).
+// the summaries, which hold as much) is set for: 1024 threads for D3Q19 (64
+// registers), 768 for D3Q27 (80).  Measured (marks and summaries of a cavity,
+// D3Q19 / prism with cubic interpolation, D3Q27): 0.91 / 17.8 ms with 768 / 512
+// threads, 0.88 / 16.9 with these, 0.94 / 17.1 with 1152 / 896 (spills).
 template <int Q, class T, int THREADS>
 constexpr int average_min_ctas() {
   return (Q == 9 ? 1024 : (sizeof(T) == 8 ? 384 : (Q == 27 ? 768 : 1024))) / THREADS;
@@ -937,40 +936,69 @@ constexpr size_t persist_smem_bytes() {
 
 // ================================================ whole blocks, read only
 // The kernels below read the pre-collision populations of whole blocks by
-// x-rows (gather_row): a warp per block in 3D, two blocks per warp in 2D.
-template <int D, class T>
+// x-rows (gather_row): a warp per block in 3D (FP64: two, a cell per thread, see
+// row_cells), two blocks per warp in 2D.
+template <int D, class T, int V_ = row_cells<D, T>()>
 struct BlockRows {
-  static constexpr int V = D == 3 ? 2 : 1;
+  static constexpr int V = V_;
   static constexpr int TPB = Block<D>::M / V;
+  static constexpr int LPR = TPB < 32 ? TPB : 32;   // lanes that share a staged row
   static constexpr int NCODE = D == 2 ? 9 : 27;
   static constexpr int BPC = 128 / TPB;     // blocks of a CTA of 128 threads
   struct Shared {
-    int32_t nb[BPC][NCODE];
-    uint64_t sm[BPC][NCODE];
+    int32_t nb[128 / LPR][NCODE];
+    uint64_t sm[128 / LPR][NCODE];
   };
 };
 
-// Populations of the V cells of this thread of block b (`slot` of its CTA).
-template <int D, int Q, class T>
-__device__ __forceinline__ void read_rows(Vec<T, BlockRows<D, T>::V> (&g)[Q], const T* f, int b,
-                                          int slot, const RowPos<D, BlockRows<D, T>::V>& pos,
-                                          typename BlockRows<D, T>::Shared& s,
+// CTAs of 128 threads per SM the register budget of the criterion and of the
+// export of moments is set for.  FP64, criterion and its synchronisation: 24^3
+// cavity, one level, D3Q27 36.5 us (41.9 with two cells per thread), 96^3 box,
+// D3Q19 167 us (173 with two), 170 with 768 threads for 640; 1024^2 box 108 us
+// with 1536 threads, 109 with 1280, 114 with 1024.
+template <int Q, class T>
+constexpr int read_min_ctas() {
+  return (Q == 9 ? 1536 : (sizeof(T) == 8 ? (Q == 27 ? 512 : 640) : (Q == 27 ? 768 : 1024))) / 128;
+}
+
+// Populations of the V cells of this thread of block b.
+template <int D, int Q, class T, int V>
+__device__ __forceinline__ void read_rows(Vec<T, V> (&g)[Q], const T* f, int b,
+                                          const RowPos<D, V>& pos,
+                                          typename BlockRows<D, T, V>::Shared& s,
                                           const int32_t* __restrict__ nbr,
                                           const uint64_t* __restrict__ solidmask) {
-  using B = BlockRows<D, T>;
-  const int flags = stage_block<D, B::TPB, true>(s.nb[slot], s.sm[slot], b, threadIdx.x % B::TPB,
-                                                 block_lanes<B::TPB>(), nbr, solidmask, nullptr);
-  gather_row<D, Q, T, B::V, true, true, false>(g, f, b, pos, s.nb[slot], s.sm[slot],
-                                               flags & BF_SOLID);
+  using B = BlockRows<D, T, V>;
+  const int row = threadIdx.x / B::LPR;
+  const int flags = stage_block<D, B::LPR, true>(s.nb[row], s.sm[row], b, threadIdx.x % B::LPR,
+                                                 block_lanes<B::LPR>(), nbr, solidmask, nullptr);
+  gather_row<D, Q, T, V, true, true, false>(g, f, b, pos, s.nb[row], s.sm[row], flags & BF_SOLID);
+}
+
+// The TPB threads of a block meet (`slot`: of the CTA).
+template <int TPB>
+__device__ __forceinline__ void block_sync(int slot) {
+  if constexpr (TPB > 32) asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(TPB) : "memory");
+  else __syncwarp(block_lanes<TPB>());
 }
 
 // Block-local first-order difference of a value along AXIS (forward, backward
-// at the last cell) for the V cells of a thread; val: the thread's values.
+// at the last cell) for the V cells of a thread; val: the thread's values.  The
+// neighbour's value comes by a shuffle, or, in blocks of more than a warp, from
+// `all`, the values of the block in shared memory.
 template <int D, int V, int AXIS, class R>
 __device__ __forceinline__ void block_diff(R (&out)[V], const R (&val)[V],
-                                           const RowPos<D, V>& pos, unsigned lanes) {
+                                           const RowPos<D, V>& pos, unsigned lanes, const R* all) {
   const int lane = threadIdx.x & 31;
-  if constexpr (AXIS == 0) {
+  // a - b or b - a, one subtraction (an FP64 one is a 64-cycle instruction)
+  auto minus = [](bool plain, R a, R b) { return (plain ? a : b) - (plain ? b : a); };
+  if constexpr (Block<D>::M / V > 32) {
+    static_assert(V == 1, "a cell per thread");
+    constexpr int STEP = AXIS == 0 ? 1 : (AXIS == 1 ? 4 : 16);
+    const int at = AXIS == 0 ? pos.i0 : (AXIS == 1 ? Block<D>::cj(pos.l0) : Block<D>::ck(pos.l0));
+    const R o = all[pos.l0 + (at == 3 ? -STEP : STEP)];
+    out[0] = minus(at == 3, val[0], o);
+  } else if constexpr (AXIS == 0) {
     if constexpr (V == 2) {
       const R next = __shfl_sync(lanes, val[0], pos.i0 == 0 ? lane + 1 : lane);
       out[0] = val[1] - val[0];
@@ -978,7 +1006,7 @@ __device__ __forceinline__ void block_diff(R (&out)[V], const R (&val)[V],
     } else {
       const bool last = pos.i0 == 3;
       const R o = __shfl_sync(lanes, val[0], last ? lane - 1 : lane + 1);
-      out[0] = last ? val[0] - o : o - val[0];
+      out[0] = minus(last, val[0], o);
     }
   } else {
     constexpr int STEP = (AXIS == 1 ? 4 : 16) / V;    // lanes between cells along the axis
@@ -986,7 +1014,7 @@ __device__ __forceinline__ void block_diff(R (&out)[V], const R (&val)[V],
 #pragma unroll
     for (int i = 0; i < V; ++i) {
       const R o = __shfl_sync(lanes, val[i], last ? lane - STEP : lane + STEP);
-      out[i] = last ? val[i] - o : o - val[i];
+      out[i] = minus(last, val[i], o);
     }
   }
 }
@@ -997,7 +1025,7 @@ __device__ __forceinline__ void block_diff(R (&out)[V], const R (&val)[V],
 // Algorithm 3 (eps < T evaluated as |w|^2 < 4^T), mark: +1 for a leaf with
 // L_des > L, -1 for a REFINED block with L_des <= L.
 template <int D, int Q, class T>
-__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
+__global__ void __launch_bounds__(128, (read_min_ctas<Q, T>()))
     k_criterion(const int32_t* __restrict__ list, int n, const T* __restrict__ f, const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
                 const int32_t* __restrict__ status, int level, int lmax, double inv_dx,
                 int n_start, int n_inc, int8_t* __restrict__ marks, double* __restrict__ w2out) {
@@ -1005,15 +1033,18 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   using R = typename S::R;
   using B = BlockRows<D, T>;
   constexpr int V = B::V;
+  constexpr bool WIDE = B::TPB > 32;         // a block takes two warps
   __shared__ typename B::Shared sh;
+  __shared__ R su[WIDE ? B::BPC : 1][D][WIDE ? Block<D>::M : 1];
+  __shared__ R sw[128 / 32];
   const int slot = threadIdx.x / B::TPB, t = threadIdx.x % B::TPB;
   const int bi = blockIdx.x * B::BPC + slot;
   if (bi >= n) return;                       // (the same for the threads of a block)
-  const unsigned lanes = block_lanes<B::TPB>();
+  const unsigned lanes = block_lanes<B::LPR>();
   const int b = __ldg(list + bi);
   const RowPos<D, V> pos(t);
   Vec<T, V> g[Q];
-  read_rows<D, Q, T>(g, f, b, slot, pos, sh, nbr, solidmask);
+  read_rows<D, Q, T, V>(g, f, b, pos, sh, nbr, solidmask);
   R u[3][V];
   static_for<0, V>([&](auto I) {
     R fl[Q];
@@ -1021,10 +1052,18 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     R rho;
     moments<D, Q>(fl, rho, u[0][I], u[1][I], u[2][I]);
   });
+  const R* all[3] = {};
+  if constexpr (WIDE) {
+    static_for<0, D>([&](auto C) {
+      su[slot][C][pos.l0] = u[C][0];
+      all[C] = su[slot][C];
+    });
+    block_sync<B::TPB>(slot);
+  }
   const R s = R(inv_dx);
   R a[V], c[V], w2[V];
-  block_diff<D, V, 0>(a, u[1], pos, lanes);
-  block_diff<D, V, 1>(c, u[0], pos, lanes);
+  block_diff<D, V, 0>(a, u[1], pos, lanes, all[1]);
+  block_diff<D, V, 1>(c, u[0], pos, lanes, all[0]);
 #pragma unroll
   for (int i = 0; i < V; ++i) w2[i] = (a[i] - c[i]) * s;
   if constexpr (D == 2) {
@@ -1032,12 +1071,12 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
     for (int i = 0; i < V; ++i) w2[i] = w2[i] * w2[i];
   } else {
     R wx[V], wy[V];
-    block_diff<D, V, 1>(a, u[2], pos, lanes);
-    block_diff<D, V, 2>(c, u[1], pos, lanes);
+    block_diff<D, V, 1>(a, u[2], pos, lanes, all[2]);
+    block_diff<D, V, 2>(c, u[1], pos, lanes, all[1]);
 #pragma unroll
     for (int i = 0; i < V; ++i) wx[i] = (a[i] - c[i]) * s;
-    block_diff<D, V, 2>(a, u[0], pos, lanes);
-    block_diff<D, V, 0>(c, u[2], pos, lanes);
+    block_diff<D, V, 2>(a, u[0], pos, lanes, all[0]);
+    block_diff<D, V, 0>(c, u[2], pos, lanes, all[2]);
 #pragma unroll
     for (int i = 0; i < V; ++i) {
       wy[i] = (a[i] - c[i]) * s;
@@ -1048,8 +1087,14 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
 #pragma unroll
   for (int i = 1; i < V; ++i) top = max(top, w2[i]);
 #pragma unroll
-  for (int off = B::TPB / 2; off > 0; off >>= 1)
+  for (int off = B::LPR / 2; off > 0; off >>= 1)
     top = max(top, __shfl_xor_sync(lanes, top, off));
+  if constexpr (WIDE) {
+    const int warp = threadIdx.x >> 5;
+    if ((threadIdx.x & 31) == 0) sw[warp] = top;
+    block_sync<B::TPB>(slot);
+    if (t == 0) top = max(top, sw[warp + 1]);
+  }
   if (t != 0) return;
   const double w2d = (double)top;
   int ldes = lmax - 1;
@@ -1088,7 +1133,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
                int level, int lmax, double inv_dx, float* __restrict__ out) {
   using S = Store<T>;
   using R = typename S::R;
-  using B = BlockRows<3, T>;
+  using B = BlockRows<3, T, 2>;
   // (rows of 68 words: 16-byte reads of eight rows touch every bank once)
   __shared__ __align__(16) float s_row[B::BPC][16][68];
   __shared__ typename B::Shared sh;
@@ -1098,7 +1143,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   const int b = __ldg(list + bi);
   const RowPos<3, 2> pos(lane);
   Vec<T, 2> g[Q];
-  read_rows<3, Q, T>(g, f, b, slot, pos, sh, nbr, solidmask);
+  read_rows<3, Q, T, 2>(g, f, b, pos, sh, nbr, solidmask);
   float u[3][2], rho[2];
   static_for<0, 2>([&](auto I) {
     R fl[Q];
@@ -1113,9 +1158,9 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   const float s = (float)inv_dx;
   float G[9][2];
   static_for<0, 3>([&](auto C) {
-    block_diff<3, 2, 0>(G[3 * C], u[C], pos, 0xffffffffu);
-    block_diff<3, 2, 1>(G[3 * C + 1], u[C], pos, 0xffffffffu);
-    block_diff<3, 2, 2>(G[3 * C + 2], u[C], pos, 0xffffffffu);
+    block_diff<3, 2, 0>(G[3 * C], u[C], pos, 0xffffffffu, (const float*)nullptr);
+    block_diff<3, 2, 1>(G[3 * C + 1], u[C], pos, 0xffffffffu, (const float*)nullptr);
+    block_diff<3, 2, 2>(G[3 * C + 2], u[C], pos, 0xffffffffu, (const float*)nullptr);
   });
   // rows: 0..8 G, 9 rho, 10..12 u, 13 |u|, 14 |w|, 15 -rho
   float (*row)[68] = s_row[slot];
@@ -1196,13 +1241,21 @@ __device__ __forceinline__ void store_doubles(double* at, const Doubles<V>& x, b
   for (int c = 0; c < V; ++c) at[c] = x.v[c];
 }
 
+// Cells per thread of the export: one; a thread holds its Q values before it
+// stores them, and with two the 126 to 178 registers of D3Q27 left too few
+// threads to keep the stores going (130,000 blocks: 296 us with two, 224 with
+// one in FP32, 338 / 253 in FP64).  D3Q19 in FP32 is faster with two (163 / 171).
 template <int D, int Q, class T>
-__global__ void __launch_bounds__(128)
+constexpr int export_cells() {
+  return D == 3 && Q == 19 && sizeof(T) == 4 ? 2 : 1;
+}
+template <int D, int Q, class T>
+__global__ void __launch_bounds__(128, D == 2 || export_cells<D, Q, T>() == 2 ? 0 : (sizeof(T) == 8 ? 6 : 8))
     k_export_f(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
                const T* __restrict__ fb, unsigned cur, const int32_t* __restrict__ level,
                const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
                double* __restrict__ out, bool wide) {
-  using B = BlockRows<D, T>;
+  using B = BlockRows<D, T, export_cells<D, Q, T>()>;
   constexpr int M = Block<D>::M, V = B::V;
   __shared__ typename B::Shared sh;
   const int slot = threadIdx.x / B::TPB, t = threadIdx.x % B::TPB;
@@ -1218,7 +1271,7 @@ __global__ void __launch_bounds__(128)
     return;
   }
   Vec<T, V> g[Q];
-  read_rows<D, Q, T>(g, ((cur >> L) & 1u) ? fb : fa, b, slot, pos, sh, nbr, solidmask);
+  read_rows<D, Q, T, V>(g, ((cur >> L) & 1u) ? fb : fa, b, pos, sh, nbr, solidmask);
   static_for<0, Q>([&](auto P) {
     Doubles<V> x;
 #pragma unroll
@@ -1247,7 +1300,7 @@ __global__ void k_import_f(int64_t cap, int64_t b0, int64_t nb, T* __restrict__ 
 }
 
 template <int D, int Q, class T>
-__global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
+__global__ void __launch_bounds__(128, (read_min_ctas<Q, T>()))
     k_export_rho_u(int64_t cap, int64_t b0, int64_t nb, const T* __restrict__ fa,
                    const T* __restrict__ fb, unsigned cur, const int32_t* __restrict__ level,
                    const int32_t* __restrict__ nbr, const uint64_t* __restrict__ solidmask,
@@ -1266,7 +1319,7 @@ __global__ void __launch_bounds__(128, (average_min_ctas<Q, T, 128>()))
   double v[V][1 + D] = {};
   if (L >= 0) {
     Vec<T, V> g[Q];
-    read_rows<D, Q, T>(g, ((cur >> L) & 1u) ? fb : fa, b, slot, pos, sh, nbr, solidmask);
+    read_rows<D, Q, T, V>(g, ((cur >> L) & 1u) ? fb : fa, b, pos, sh, nbr, solidmask);
     static_for<0, V>([&](auto I) {
       R fl[Q];
       static_for<0, Q>([&](auto P) { fl[P] = S::template load<D, Q, P>(g[P].v[I]); });
@@ -1637,7 +1690,7 @@ struct Launch {
   static void export_f(cudaStream_t s, int64_t cap, int64_t b0, int64_t nb, const void* fa,
                        const void* fb, unsigned cur, const int32_t* level, const int32_t* nbr,
                        const uint64_t* sm, double* out) {
-    k_export_f<D, Q, T><<<grid_for(nb, BlockRows<D, T>::BPC), 128, 0, s>>>(
+    k_export_f<D, Q, T><<<grid_for(nb, BlockRows<D, T, export_cells<D, Q, T>()>::BPC), 128, 0, s>>>(
         cap, b0, nb, (const T*)fa, (const T*)fb, cur, level, nbr, sm, out, (uintptr_t)out % 16 == 0);
   }
   static void import_f(cudaStream_t s, int64_t cap, int64_t b0, int64_t nb, void* fa, void* fb,
