@@ -636,13 +636,10 @@ __device__ __forceinline__ int stage_block(int32_t* s_nb, uint64_t* s_sm, int b,
 }
 
 // The links of cell l that leave through a moving wall or an outlet: their
-// stored value takes the wall's rule.  Out of line: few blocks have one.  The
-// values go through an array of their own, which lives in local memory:
-// handing f itself over makes every cell of every block store its f there
-// (1.6x the write traffic of the level, measured).
+// stored value takes the wall's rule.
 template <int D, int Q, bool SHIFTED, class R>
-__device__ __noinline__ void wall_links_of(R* f, const Relax<D, Q, SHIFTED, R> r, int l,
-                                           const int32_t* nb, const FaceParams& faces) {
+__device__ __forceinline__ void wall_links_in(R* f, const Relax<D, Q, SHIFTED, R>& r, int l,
+                                              const int32_t* nb, const FaceParams& faces) {
   static_for<1, Q>([&](auto P) {
     constexpr int p = P;
     const int to = nb[link_entry<D, Q, p>(g_tgt_geo<D, Q>, l) & 31];
@@ -650,13 +647,29 @@ __device__ __noinline__ void wall_links_of(R* f, const Relax<D, Q, SHIFTED, R> r
   });
 }
 
+// 3D: out of line, few blocks have such a link.  The values go through an array
+// of their own, which lives in local memory: handing f itself over makes every
+// cell of every block store its f there (1.6x the write traffic of the level,
+// measured).  2D: in line; a launch is as long as its slowest block (80x100
+// FP32 cavity, one level: 7.7 us per launch out of line, 7.2 in
+// line, of which 4.3 without walls).
+template <int D, int Q, bool SHIFTED, class R>
+__device__ __noinline__ void wall_links_of(R* f, const Relax<D, Q, SHIFTED, R> r, int l,
+                                           const int32_t* nb, const FaceParams& faces) {
+  wall_links_in<D, Q, SHIFTED, R>(f, r, l, nb, faces);
+}
+
 template <int D, int Q, bool SHIFTED, class R>
 __device__ __forceinline__ void wall_links(R (&f)[Q], const Relax<D, Q, SHIFTED, R>& r, int l,
                                            const int32_t* nb, const FaceParams& faces) {
-  R w[Q];
-  static_for<0, Q>([&](auto P) { w[P] = f[P]; });
-  wall_links_of<D, Q, SHIFTED, R>(w, r, l, nb, faces);
-  static_for<0, Q>([&](auto P) { f[P] = w[P]; });
+  if constexpr (D == 2) {
+    wall_links_in<D, Q, SHIFTED, R>(f, r, l, nb, faces);
+  } else {
+    R w[Q];
+    static_for<0, Q>([&](auto P) { w[P] = f[P]; });
+    wall_links_of<D, Q, SHIFTED, R>(w, r, l, nb, faces);
+    static_for<0, Q>([&](auto P) { f[P] = w[P]; });
+  }
 }
 template <int D, int Q, bool SHIFTED>
 __device__ __forceinline__ void wall_links(F2 (&f)[Q], const Relax<D, Q, SHIFTED, F2>& r, int l,
