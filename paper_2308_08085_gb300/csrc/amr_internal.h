@@ -96,9 +96,9 @@ struct Instance {
   // are not chained at all now); 128^2 FP32 cavity, all launches small: 1.91 -> 1.61).
   // FP64 launches are bound by the arithmetic of the busiest SM, and a dependent
   // launch is placed around what its predecessor still holds, unevenly: none of
-  // a 3D FP64 coarse step is chained (29 forests of 24^3 to 128x32x16 root
-  // cells: 0 to 16 % slower), and all of a 2D one or nothing, by its cell
-  // updates (273 forests: up to 2^18 updates 7 % faster in the mean and at most
+  // a 3D FP64 coarse step is chained (28 forests of 24^3 to 128x32x16 root
+  // cells: 4 % slower in the mean, up to 16 %), and all of a 2D one or nothing, by its cell
+  // updates (273 forests: up to 2^18 updates 9 % faster in the mean and at most
   // 1 % slower, from there to 390,000 8 % either way, above up to 30 % slower).
   static constexpr int64_t kChainCells = int64_t(1) << 17;
   static constexpr int64_t kChainUpdates64 = int64_t(1) << 18;
