@@ -121,8 +121,8 @@ typedef struct {
                               least the blocks of one warp); 5: 128 cells with
                               128 more resident threads per SM (tighter
                               register budget); 0 (default): 256 cells in 3D,
-                              64 in 2D (128 above 2^18 cells) and in 3D FP64,
-                              32 in 2D FP64                                  */
+                              64 for FP64 and D3Q27 FP32; 64 in 2D (128 above
+                              2^18 cells), 32 in 2D FP64                     */
   double refine_dist;      /* distance refinement (Section 4.4): a leaf on level
                               L within refine_dist / 2^L (physical units) of a
                               target is marked for refinement; 0 = off        */

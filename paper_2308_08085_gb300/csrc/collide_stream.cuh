@@ -433,19 +433,23 @@ __device__ __forceinline__ Vec<T, V> ld_vec(const T* p) {
 // its rate: two warps per block reach it with half the blocks (coarse steps of
 // cavities and prisms, one against two: 24^3 16.4 / 26.6 us, 24^3 with two extra
 // levels 658 / 773, 64^3 with one 579 / 612, 128x32x16 prism with three 3461 /
-// 3632; none slower).  2D: one; the meshes are small and latency counts (128^2
-// cavity, FP32, 20 coarse steps: 1.9 / 2.2 / 3.0 ms with 1 / 2 / 4).
-template <int D, class T>
+// 3632; none slower).  D3Q27 in FP32: one; two leave room for 20 warps of 96
+// registers, one for 32 of 64 (prism of 2.6 million finest blocks 24,830 / 24,050
+// MLUPS, 128x32x32 prism, cubic, five coarse steps 14.1 / 14.7 ms, 48x24x16 prism
+// with one level 40 / 53 us).  2D: one; the meshes are small and latency counts
+// (128^2 cavity, FP32, 20 coarse steps: 1.9 / 2.2 / 3.0 ms with 1 / 2 / 4).
+template <int D, int Q, class T>
 constexpr int row_cells() {
-  return D == 2 || sizeof(T) == 8 ? 1 : 2;
+  return D == 2 || sizeof(T) == 8 || (Q == 27 && sizeof(T) == 4) ? 1 : 2;
 }
 
 // Threads of a CTA that holds `cells` cells, V per thread (at least a warp), and
 // the CTAs per SM its register budget is set for: 896 threads for D3Q19 in 32 bits and
 // less (72 registers; the cavity above takes 37.0 / 36.1 / 36.3 ms with 768 /
-// 896 / 1024), 640 for D3Q27 (96 registers; 13.8 ms against 15.4 with 768 for
-// five coarse steps of the 128x32x32 prism in FP16), fewer for FP64, whose
-// arithmetic saturates with few warps.
+// 896 / 1024), 1024 for D3Q27 in FP32 (a cell per thread), 640 in 16 bits (96
+// registers; 13.8 ms against 15.4 with 768 for five coarse steps of the
+// 128x32x32 prism in FP16), fewer for FP64, whose arithmetic saturates with few
+// warps.
 template <int V>
 constexpr int row_threads(int cells) {
   return cells / V < 32 ? 32 : cells / V;
@@ -453,7 +457,7 @@ constexpr int row_threads(int cells) {
 template <int Q, class T, int THREADS, bool DENSE = false>
 constexpr int row_min_ctas() {
   const int threads = (Q == 9 ? 1024 : (sizeof(T) == 8 ? (Q == 19 ? 512 : 384)
-                                                       : (Q == 19 ? 896 : 640))) +
+                                                       : (Q == 19 ? 896 : (sizeof(T) == 4 ? 1024 : 640)))) +
                       (DENSE ? 128 : 0);
   return threads / THREADS > 0 ? threads / THREADS : 1;
 }
@@ -909,7 +913,7 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
                      const uint64_t* __restrict__ cellmask, const __grid_constant__ Exchange ex) {
   using R = typename Store<T>::R;
   constexpr int M = Block<D>::M;
-  constexpr int V = row_cells<D, T>();
+  constexpr int V = row_cells<D, Q, T>();
   constexpr int TPB = M / V;                // threads of a block
   constexpr int LPR = TPB < 32 ? TPB : 32;  // lanes that share a staged row
   constexpr int NCODE = D == 2 ? 9 : 27;

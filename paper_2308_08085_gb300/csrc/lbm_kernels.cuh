@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
     k_collide_stream_batch(const uint32_t* __restrict__ items, int n,
                            const InstDesc* __restrict__ descs, int level, int which_in) {
   using R = typename Store<T>::R;
-  constexpr int V = row_cells<D, T>();
+  constexpr int V = row_cells<D, Q, T>();
   constexpr int TPB = Block<D>::M / V, LPR = TPB < 32 ? TPB : 32;
   constexpr int BPC = THREADS / TPB;
   __shared__ int32_t s_nb[THREADS / LPR][D == 2 ? 9 : 27];
@@ -910,10 +910,10 @@ __global__ void __launch_bounds__(THREADS, (persist_min_ctas<Q, T, THREADS>()))
       // a cell per thread where two would leave half of the warps without work
       // (the batch above, CTAs of 256 with tiles of one block: 5.1 ms against
       // 3.3 with this and the budget)
-      if (row_cells<D, T>() == 1 || 2 * nblk * 32 <= THREADS)
+      if (row_cells<D, Q, T>() == 1 || 2 * nblk * 32 <= THREADS)
         persist_collide<D, Q, T, THREADS, 1>(d, items + first, nblk, level, win, s_nb);
       else
-        persist_collide<D, Q, T, THREADS, row_cells<D, T>()>(d, items + first, nblk, level, win,
+        persist_collide<D, Q, T, THREADS, row_cells<D, Q, T>()>(d, items + first, nblk, level, win,
                                                              s_nb);
     } else if (op == PH_INTERP) {
       persist_interp<D, Q, T, THREADS>(d, items, ni, tile, level, win, wch, sF, s_rows);
@@ -938,7 +938,7 @@ constexpr size_t persist_smem_bytes() {
 // The kernels below read the pre-collision populations of whole blocks by
 // x-rows (gather_row): a warp per block in 3D (FP64: two, a cell per thread, see
 // row_cells), two blocks per warp in 2D.
-template <int D, class T, int V_ = row_cells<D, T>()>
+template <int D, class T, int V_ = D == 2 || sizeof(T) == 8 ? 1 : 2>
 struct BlockRows {
   static constexpr int V = V_;
   static constexpr int TPB = Block<D>::M / V;
@@ -1561,7 +1561,7 @@ struct Launch {
   // cells per CTA.  2D meshes are small: CTAs of one or two warps spread them
   // over the SMs (an SM executes one FP64 warp instruction per 19 cycles; the
   // 64^2 FP64 cavity took 2.20 ms with 256 cells per CTA, 1.66 with 32)
-  static constexpr int kAutoCells = D == 3 ? (sizeof(T) == 8 ? 64 : 256)
+  static constexpr int kAutoCells = D == 3 ? (row_cells<D, Q, T>() == 1 ? 64 : 256)
                                            : (sizeof(T) == 8 ? 32 : 64);
   // ... 2D FP32 launches above this many cells: CTAs of 128 (one level, us per
   // step with 64 / 128 cells: 512^2 8.3 / 8.3, 768^2 12.4 / 10.4, 1024^2 20.6 /
@@ -1582,7 +1582,7 @@ struct Launch {
   static void one_pass(cudaStream_t s, const int32_t* list, int n, const void* fin, void* fout,
                        const int32_t* nbr, const uint64_t* sm, const StepParams& prm,
                        const uint64_t* gm, const Exchange* xchg) {
-    constexpr int V = row_cells<D, T>(), THREADS = row_threads<V>(CELLS);
+    constexpr int V = row_cells<D, Q, T>(), THREADS = row_threads<V>(CELLS);
     constexpr int MIN = row_min_ctas<Q, T, THREADS, DENSE>();
     const T* in = (const T*)fin;
     T* out = (T*)fout;
@@ -1760,7 +1760,7 @@ struct Launch {
   template <int CELLS>
   static void batch_cells(cudaStream_t s, const uint32_t* items, int n, const InstDesc* descs,
                           int level, int which_in) {
-    constexpr int V = row_cells<D, T>(), THREADS = row_threads<V>(CELLS);
+    constexpr int V = row_cells<D, Q, T>(), THREADS = row_threads<V>(CELLS);
     k_collide_stream_batch<D, Q, T, THREADS>
         <<<grid_for(n, THREADS * V / M), THREADS, 0, s>>>(items, n, descs, level, which_in);
   }
