@@ -446,7 +446,7 @@ constexpr int row_cells() {
 // Threads of a CTA that holds `cells` cells, V per thread (at least a warp), and
 // the CTAs per SM its register budget is set for: 896 threads for D3Q19 in 32 bits and
 // less (72 registers; the cavity above takes 37.0 / 36.1 / 36.3 ms with 768 /
-// 896 / 1024), 1024 for D3Q27 in FP32 (a cell per thread), 640 in 16 bits (96
+// 896 / 1024), 1024 for D3Q27 with a cell per thread, 640 with two (96
 // registers; 13.8 ms against 15.4 with 768 for five coarse steps of the
 // 128x32x32 prism in FP16), fewer for FP64, whose arithmetic saturates with few
 // warps.
@@ -454,10 +454,10 @@ template <int V>
 constexpr int row_threads(int cells) {
   return cells / V < 32 ? 32 : cells / V;
 }
-template <int Q, class T, int THREADS, bool DENSE = false>
+template <int Q, class T, int V, int THREADS, bool DENSE = false>
 constexpr int row_min_ctas() {
   const int threads = (Q == 9 ? 1024 : (sizeof(T) == 8 ? (Q == 19 ? 512 : 384)
-                                                       : (Q == 19 ? 896 : (sizeof(T) == 4 ? 1024 : 640)))) +
+                                                       : (Q == 19 ? 896 : (V == 1 ? 1024 : 640)))) +
                       (DENSE ? 128 : 0);
   return threads / THREADS > 0 ? threads / THREADS : 1;
 }
@@ -904,7 +904,8 @@ __device__ __forceinline__ void interp_rows(const typename Store<T>::R* rc, int 
 // cells to its children's interpolation, need no CTA barrier.  With one cell
 // per thread in 3D a block takes two warps: each stages the row for itself, and
 // the CTA, which then holds one block, meets before the interpolation.
-template <int D, int Q, class T, bool SOLID, int THREADS, int MIN_CTAS, bool GHOST_IN, bool XCHG>
+template <int D, int Q, class T, bool SOLID, int V, int THREADS, int MIN_CTAS, bool GHOST_IN,
+          bool XCHG>
 __global__ void __launch_bounds__(THREADS, MIN_CTAS)
     k_collide_stream(const int32_t* __restrict__ list, int n, const T* gin,
                      T* gout, const int32_t* __restrict__ nbr,
@@ -913,7 +914,6 @@ __global__ void __launch_bounds__(THREADS, MIN_CTAS)
                      const uint64_t* __restrict__ cellmask, const __grid_constant__ Exchange ex) {
   using R = typename Store<T>::R;
   constexpr int M = Block<D>::M;
-  constexpr int V = row_cells<D, Q, T>();
   constexpr int TPB = M / V;                // threads of a block
   constexpr int LPR = TPB < 32 ? TPB : 32;  // lanes that share a staged row
   constexpr int NCODE = D == 2 ? 9 : 27;

@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(64, (average_min_ctas<Q, T, 64>()))
 // instance's buffers, tables and per-level factors come from its descriptor.
 // The same step as k_collide_stream (no solid cells in a batch).
 template <int D, int Q, class T, int THREADS>
-__global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, THREADS>()))
+__global__ void __launch_bounds__(THREADS, (row_min_ctas<Q, T, row_cells<D, Q, T>(), THREADS>()))
     k_collide_stream_batch(const uint32_t* __restrict__ items, int n,
                            const InstDesc* __restrict__ descs, int level, int which_in) {
   using R = typename Store<T>::R;
@@ -1567,6 +1567,10 @@ struct Launch {
   // step with 64 / 128 cells: 512^2 8.3 / 8.3, 768^2 12.4 / 10.4, 1024^2 20.6 /
   // 16.6, 2048^2 71.8 / 63.6, 3072^2 153.8 / 134.9)
   static constexpr int64_t kWideCells = int64_t(1) << 18;
+  // ... D3Q27 FP32 launches of more blocks than this without solid cells: two
+  // cells per thread, 256 per CTA (192^3 box: 244 us per step, 261 with one; 64^3
+  // cavity with an extra level, launches of up to 13,000 blocks: 102 and 97)
+  static constexpr int kLargeQ27 = 1 << 14;
 
   static int setup() {
     int dev = 0, sms = 0;
@@ -1578,12 +1582,12 @@ struct Launch {
 
   // CELLS cells per CTA (at least the blocks of a warp); XCHG:
   // instantiated for launches with exchanging parents as well
-  template <bool SOLID, int CELLS, bool XCHG, bool DENSE = false>
+  template <bool SOLID, int CELLS, bool XCHG, int V = row_cells<D, Q, T>(), bool DENSE = false>
   static void one_pass(cudaStream_t s, const int32_t* list, int n, const void* fin, void* fout,
                        const int32_t* nbr, const uint64_t* sm, const StepParams& prm,
                        const uint64_t* gm, const Exchange* xchg) {
-    constexpr int V = row_cells<D, Q, T>(), THREADS = row_threads<V>(CELLS);
-    constexpr int MIN = row_min_ctas<Q, T, THREADS, DENSE>();
+    constexpr int THREADS = row_threads<V>(CELLS);
+    constexpr int MIN = row_min_ctas<Q, T, V, THREADS, DENSE>();
     const T* in = (const T*)fin;
     T* out = (T*)fout;
     Exchange ex{};
@@ -1591,7 +1595,7 @@ struct Launch {
     auto launch = [&](auto ghost, auto parents) {
       constexpr bool G = decltype(ghost)::value, X = decltype(parents)::value;
       const int grid = grid_for(n, THREADS * V / M);
-      launch_chained(k_collide_stream<D, Q, T, SOLID, THREADS, MIN, G, X>, prm.chained, grid,
+      launch_chained(k_collide_stream<D, Q, T, SOLID, V, THREADS, MIN, G, X>, prm.chained, grid,
                      THREADS, s, list, n, in, out, nbr, sm, prm, gm, ex);
     };
     if constexpr (XCHG) {
@@ -1616,12 +1620,18 @@ struct Launch {
       case 3: one_pass<SOLID, 128, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 4: one_pass<SOLID, 64, false>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr); break;
       case 5:
-        one_pass<SOLID, 128, false, true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr);
+        one_pass<SOLID, 128, false, row_cells<D, Q, T>(), true>(s, list, n, fin, fout, nbr, sm, prm, gm, nullptr);
         break;
       default:
         if constexpr (D == 2 && sizeof(T) == 4) {
           if ((int64_t)n * M > kWideCells) {
             one_pass<SOLID, 128, true>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
+            break;
+          }
+        }
+        if constexpr (Q == 27 && sizeof(T) == 4 && !SOLID) {
+          if (n > kLargeQ27) {
+            one_pass<SOLID, 256, true, 2>(s, list, n, fin, fout, nbr, sm, prm, gm, x);
             break;
           }
         }
